@@ -166,7 +166,9 @@ hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule);
  * stack entries than the shape has is reported as HCC_ERR_STACK_OVERFLOW by
  * hcc_sync (its record is a miss): a binary layout needs at most the BVH's
  * depth (hcc_bvh_info), the 4-ary layout up to three entries per 4-ary
- * level.  Results do not depend on the shape otherwise.  (0, 0) restores
+ * level.  (The compact nodes that traces prefer, see hcc_bvh_layout, are walked
+ * only where no ray can need more entries than the shape has.)  Results do not
+ * depend on the shape otherwise.  (0, 0) restores
  * the default (128, HCC_TRACE_STACK).  Errors: INVALID_ARG for any other
  * pair.
  */
@@ -227,6 +229,14 @@ typedef enum hcc_bvh_layout {
                               the largest surface area replaced by its two children until four are
                               held), the children's exact FP32 boxes as rows of four per bound */
 } hcc_bvh_layout;
+
+/* Besides the nodes of its layout every BVH holds compact 4-ary nodes (64 bytes,
+ * 16-bit bounds on a grid over the whole scene, rounded outward), unless its
+ * boxes do not suit them: a scene wider than 1e9 or narrower than 1e-9 units, or
+ * boxes so small against it that the grid would add a fifth to their surface.
+ * Traces (single, batches, servers) walk the compact nodes where their deepest
+ * stack fits the trace's; the layout's nodes are what they walk otherwise, what
+ * hcc_trace_counts counts and what the prefix path code reads. */
 
 /* hcc_bvh_upload with a choice of node layout.  Every layout gives the same
  * hits (boxes only decide which triangles are tested, and every box holds
@@ -419,8 +429,8 @@ hcc_status hcc_gather(hcc_ctx *ctx, const hcc_rays *in, const uint32_t *perm, co
 
 /*
  * Closest hit (any_hit = 0) or any hit (any_hit != 0) of every ray against
- * the BVH's triangles by stack-based traversal of the quantised BVH2 and
- * the Moller-Trumbore test (two-sided, no epsilon, hit when tmin < t <
+ * the BVH's triangles by stack-based traversal (hcc_bvh_layout) and the
+ * Moller-Trumbore test (two-sided, no epsilon, hit when tmin < t <
  * tmax).  Closest hit = smallest t, ties to the lower triangle id; it does
  * not depend on traversal order.  Any hit reports some hit of the ray.
  * Result of ray j goes to hits[j], or to hits[scatter[j]] when scatter is
@@ -447,7 +457,8 @@ hcc_status hcc_trace_sorted(hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *ra
 
 /*
  * Diagnostic (never on the timed path): trace like hcc_trace (perm NULL) or
- * hcc_trace_sorted (perm given) and count, over all rays: counts[0] internal
+ * hcc_trace_sorted (perm given), through the nodes of the BVH's layout, and
+ * count, over all rays: counts[0] internal
  * node visits, counts[1] triangle tests, counts[2] warp-level node steps
  * (loop iterations of a warp in which any lane visits a node), counts[3]
  * warp-level leaf steps.  counts[0] / (32 counts[2]) is the warp execution

@@ -10,8 +10,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <future>
 #include <new>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include "hcc_internal.cuh"
@@ -61,6 +63,10 @@ struct hcc_bvh {
     uint32_t *d_prim_rec = nullptr;  // triangle id -> record index
     uint32_t num_nodes = 0, num_internal = 0, num_tris = 0, depth = 0;
     uint32_t root_ref = 0;
+    // compact nodes for the traces (NULL where the scene does not suit them)
+    uint4 *d_compact = nullptr;
+    uint32_t compact_root = 0, compact_stack = 0xFFFFFFFFu;
+    hcc::Grid grid = {};
     // exact tree kept on the host for cut selection
     std::vector<float> lo, hi;
     std::vector<int32_t> left, right;
@@ -83,6 +89,7 @@ struct hcc_batch {
     int device = 0;
     int layout = 0;
     uint32_t num_scenes = 0;
+    uint32_t compact_stack = 0xFFFFFFFFu;  // stack entries the compact nodes of every scene fit in
     uint32_t scene_bits = 0;  // bits above the key that hold the scene index
     std::vector<uint64_t> offsets;
     hcc::SceneDesc *d_scenes = nullptr;
@@ -315,13 +322,17 @@ struct HadHeap {
 namespace hcc {
 
 // Device views of the handles for the serving loop (serve.cu).
-void bvh_view(const hcc_bvh *b, SceneDesc *out, int *layout, int *device) {
+void bvh_view(const hcc_bvh *b, SceneDesc *out, int *layout, uint32_t *compact_stack, int *device) {
     std::memset(out, 0, sizeof *out);
     out->nodes = b->d_nodes;
     out->tris = b->d_tris;
     out->prim_rec = b->d_prim_rec;
     out->root_ref = b->root_ref;
     out->num_tris = b->num_tris;
+    out->cnodes = b->d_compact;
+    out->croot = b->compact_root;
+    out->grid = b->grid;
+    *compact_stack = b->compact_stack;
     for (int a = 0; a < 3; ++a) {
         out->lo[a] = b->lo[a];
         out->ext[a] = b->hi[a] - b->lo[a];
@@ -343,6 +354,29 @@ void cut_view(const hcc_cut *c, const float4 **boxes, uint32_t *on_device, int *
 static unsigned long long *trace_work(const hcc_ctx *ctx, int any_hit) {
     const bool refill = ctx->schedule == HCC_TRACE_REFILL || (ctx->schedule == HCC_TRACE_AUTO && !any_hit);
     return refill ? ctx->d_work : nullptr;
+}
+
+// What the traces of one BVH share: the scene, the rays and the context's settings.
+static TraceArgs trace_args(const hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *rays, int any_hit) {
+    TraceArgs a;
+    a.nodes = bvh->d_nodes;
+    a.layout = bvh->layout;
+    a.tris = bvh->d_tris;
+    a.root_ref = bvh->root_ref;
+    a.cnodes = bvh->d_compact;
+    a.croot = bvh->compact_root;
+    a.cstack = bvh->compact_stack;
+    a.grid = bvh->grid;
+    a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
+    a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
+    a.rs = ray_rs(rays);
+    a.rec = ray_rec(rays);
+    a.n = rays->n;
+    a.err = ctx->d_err;
+    a.work = trace_work(ctx, any_hit);
+    a.block = (int)ctx->trace_block;
+    a.stack = (int)ctx->trace_stack;
+    return a;
 }
 
 // ================================================================== C ABI
@@ -580,6 +614,129 @@ static uint32_t collapse_wide(const hcc_bvh_desc *d, std::vector<uint32_t> &word
     return (uint32_t)order.size();
 }
 
+// Compact 4-ary nodes of a validated BVH2 (boxes with lo <= hi): the collapse
+// of collapse_wide, numbered so that the internal children of a node are
+// neighbours and subtrees stay together.  usable is false where the boxes do not
+// suit the grid: not finite, a scene of extreme size, or boxes so small against
+// the scene that rounding them outward multiplies their summed surface, and with
+// it the expected node visits, by more than COMPACT_AREA (the compact walk is
+// 1.25 to 1.4 times as fast as the others' at the same visits).
+struct CompactNodes {
+    bool usable = false;
+    std::vector<uint32_t> words;
+    Grid grid = {};
+    uint32_t root = 0;
+    uint32_t stack = 0;  // most subtrees a traversal can have pending
+};
+constexpr double COMPACT_AREA = 1.2;
+
+static CompactNodes compact_nodes(const hcc_bvh_desc *d, uint32_t num_internal) {
+    CompactNodes c;
+    const uint32_t N = d->num_nodes;
+    auto leaf_ref = [&](int32_t k) { return REF_LEAF | ((d->count[k] - 1u) << 29) | d->first[k]; };
+    float lo[3], hi[3];
+    for (int a = 0; a < 3; ++a) lo[a] = hi[a] = d->lo[a];
+    bool finite = true;
+    for (uint32_t k = 0; k < N; ++k)
+        for (int a = 0; a < 3; ++a) {
+            const float l = d->lo[3 * (size_t)k + a], h = d->hi[3 * (size_t)k + a];
+            finite = finite && std::fabs(l) < 1e30f && std::fabs(h) < 1e30f;  // false for NaN
+            lo[a] = std::min(lo[a], l);
+            hi[a] = std::max(hi[a], h);
+        }
+    if (!finite) return c;
+    const float widest = std::max(hi[0] - lo[0], std::max(hi[1] - lo[1], hi[2] - lo[2]));
+    if (!(widest > 1e-9f && widest < 1e9f)) return c;
+    for (int a = 0; a < 3; ++a) {
+        // a flat axis takes the widest axis's scale
+        const float ext = std::max(hi[a] - lo[a], widest * 1e-6f);
+        c.grid.lo[a] = lo[a];
+        c.grid.scale[a] = GRID_SPAN / ext;
+    }
+    if (d->left[0] < 0) {  // a leaf root: no node is read
+        c.words.assign(16, 0u);
+        c.root = leaf_ref(0);
+        c.usable = true;
+        return c;
+    }
+    const Grid &g = c.grid;
+    auto grid_bits = [&](float x, int a, double margin) {
+        const float v = (float)(((double)x - (double)g.lo[a]) * (double)g.scale[a] + (double)GRID_ORIGIN + margin);
+        uint32_t b;
+        std::memcpy(&b, &v, 4);
+        return b;
+    };
+    const float inv[3] = {1.0f / g.scale[0], 1.0f / g.scale[1], 1.0f / g.scale[2]};
+    auto decoded = [](uint32_t q) {
+        const uint32_t b = 0x40000000u | (q << 8);
+        float f;
+        std::memcpy(&f, &b, 4);
+        return f;
+    };
+    auto half_area = [](float ex, float ey, float ez) { return ex * ey + ey * ez + ez * ex; };
+    auto area = [&](int32_t k) {
+        const float *l = d->lo + 3 * (size_t)k, *h = d->hi + 3 * (size_t)k;
+        return half_area(h[0] - l[0], h[1] - l[1], h[2] - l[2]);
+    };
+    struct Todo {
+        int32_t node;
+        uint32_t at, pending;
+    };
+    std::vector<Todo> todo{{0, 0u, 0u}};
+    c.words.resize((size_t)num_internal * 16);
+    uint32_t used = 1;
+    double exact_area = 0.0, grid_area = 0.0;
+    while (!todo.empty()) {
+        const Todo t = todo.back();
+        todo.pop_back();
+        int32_t ch[4] = {d->left[t.node], d->right[t.node], -1, -1};
+        float ar[4] = {area(ch[0]), area(ch[1]), 0.0f, 0.0f};
+        int n = 2;
+        while (n < 4) {
+            int best = -1;
+            for (int i = 0; i < n; ++i)
+                if (d->left[ch[i]] >= 0 && (best < 0 || ar[i] > ar[best])) best = i;
+            if (best < 0) break;
+            const int32_t k = ch[best];
+            ch[best] = d->left[k];
+            ar[best] = area(ch[best]);
+            ch[n] = d->right[k];
+            ar[n] = area(ch[n]);
+            ++n;
+        }
+        const uint32_t pending = t.pending + (uint32_t)n - 1u;
+        c.stack = std::max(c.stack, pending);
+        uint32_t *w = &c.words[16 * (size_t)t.at];
+        for (int i = 0; i < 4; ++i) {
+            if (i >= n) {
+                w[3 * i] = w[3 * i + 1] = w[3 * i + 2] = 0x0000FFFFu;  // lo above hi
+                w[12 + i] = 0xFFFFFFFFu;
+                continue;
+            }
+            const int32_t k = ch[i];
+            float e[3];
+            for (int a = 0; a < 3; ++a) {
+                const uint32_t l = grid_bits(d->lo[3 * (size_t)k + a], a, -(double)GRID_MARGIN) >> 8;
+                const uint32_t h = (grid_bits(d->hi[3 * (size_t)k + a], a, (double)GRID_MARGIN) + 0xFFu) >> 8;
+                w[3 * i + a] = (l & 0xFFFFu) | (h << 16);
+                e[a] = (decoded(h & 0xFFFFu) - decoded(l & 0xFFFFu)) * inv[a];
+            }
+            exact_area += ar[i];
+            grid_area += half_area(e[0], e[1], e[2]);
+            if (d->left[k] < 0) {
+                w[12 + i] = leaf_ref(k);
+            } else {
+                w[12 + i] = used;
+                todo.push_back({k, used, pending});
+                ++used;
+            }
+        }
+    }
+    c.words.resize((size_t)used * 16);
+    c.usable = grid_area <= COMPACT_AREA * exact_area;
+    return c;
+}
+
 hcc_status hcc_bvh_upload(hcc_ctx *ctx, const hcc_bvh_desc *d, hcc_bvh **out) {
     return hcc_bvh_upload_layout(ctx, d, HCC_BVH_QUANTISED, out);
 }
@@ -639,6 +796,12 @@ hcc_status hcc_bvh_upload_layout(hcc_ctx *ctx, const hcc_bvh_desc *d, hcc_bvh_la
     hcc_bvh_desc nd = *d;
     nd.lo = blo.data();
     nd.hi = bhi.data();
+    // the compact nodes are built beside the rest of the upload
+    std::future<CompactNodes> building;
+    try {
+        building = std::async(std::launch::async, [&nd, &internal] { return compact_nodes(&nd, (uint32_t)internal.size()); });
+    } catch (const std::system_error &) {  // no thread to be had: built below
+    }
     std::vector<uint32_t> words;
     uint32_t num_device_nodes = (uint32_t)internal.size();
     if (layout == HCC_BVH_WIDE) {
@@ -706,6 +869,21 @@ hcc_status hcc_bvh_upload_layout(hcc_ctx *ctx, const hcc_bvh_desc *d, hcc_bvh_la
     if (e == cudaSuccess) e = cudaMemcpy(b->d_nodes, words.data(), words.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_tris, tri.data(), tri.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_prim_rec, prim_rec.data(), (size_t)T * 4, cudaMemcpyHostToDevice);
+    CompactNodes compact;
+    try {
+        compact = building.valid() ? building.get() : compact_nodes(&nd, (uint32_t)internal.size());
+    } catch (const std::bad_alloc &) {
+        hcc_bvh_destroy(b);
+        return fail(ctx, HCC_ERR_OOM, "host allocation");
+    }
+    if (compact.usable) {
+        b->compact_root = compact.root;
+        b->compact_stack = compact.stack;
+        b->grid = compact.grid;
+        if (e == cudaSuccess) e = cudaMalloc(&b->d_compact, compact.words.size() * 4);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(b->d_compact, compact.words.data(), compact.words.size() * 4, cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         hcc_bvh_destroy(b);
@@ -735,6 +913,7 @@ hcc_status hcc_bvh_destroy(hcc_bvh *b) {
         if (b->d_nodes) cudaFree(b->d_nodes);
         if (b->d_tris) cudaFree(b->d_tris);
         if (b->d_prim_rec) cudaFree(b->d_prim_rec);
+        if (b->d_compact) cudaFree(b->d_compact);
     }
     delete b;
     return HCC_OK;
@@ -1121,27 +1300,9 @@ hcc_status hcc_trace(hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *rays, int
     if (!hits || !aligned(hits, 16)) return fail(ctx, HCC_ERR_INVALID_ARG, "hits NULL or not 16-byte aligned");
     if (scatter && !aligned(scatter, 4)) return fail(ctx, HCC_ERR_INVALID_ARG, "scatter misaligned");
     DeviceGuard g(ctx->device);
-    TraceArgs a;
-    a.nodes = bvh->d_nodes;
-    a.layout = bvh->layout;
-    a.tris = bvh->d_tris;
-    a.root_ref = bvh->root_ref;
-    a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
-    a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
-    a.rs = ray_rs(rays);
-    a.rec = ray_rec(rays);
-    a.n = rays->n;
-    a.gather = nullptr;
+    TraceArgs a = trace_args(ctx, bvh, rays, any_hit);
     a.scatter = scatter;
     a.hits = reinterpret_cast<int4 *>(hits);
-    a.err = ctx->d_err;
-    a.work = trace_work(ctx, any_hit);
-    a.block = (int)ctx->trace_block;
-    a.stack = (int)ctx->trace_stack;
-    a.counts = nullptr;
-    a.scenes = nullptr;
-    a.offsets = nullptr;
-    a.num_scenes = 0;
     cudaError_t e = launch_trace(ctx->stream, a, any_hit);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "trace launch");
     return HCC_OK;
@@ -1157,27 +1318,10 @@ hcc_status hcc_trace_sorted(hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *ra
     if (!hits || !aligned(hits, 16)) return fail(ctx, HCC_ERR_INVALID_ARG, "hits NULL or not 16-byte aligned");
     if (!perm || !aligned(perm, 4)) return fail(ctx, HCC_ERR_INVALID_ARG, "perm NULL or misaligned");
     DeviceGuard g(ctx->device);
-    TraceArgs a;
-    a.nodes = bvh->d_nodes;
-    a.layout = bvh->layout;
-    a.tris = bvh->d_tris;
-    a.root_ref = bvh->root_ref;
-    a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
-    a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
-    a.rs = ray_rs(rays);
-    a.rec = ray_rec(rays);
-    a.n = rays->n;
+    TraceArgs a = trace_args(ctx, bvh, rays, any_hit);
     a.gather = perm;
     a.scatter = perm;
     a.hits = reinterpret_cast<int4 *>(hits);
-    a.err = ctx->d_err;
-    a.work = trace_work(ctx, any_hit);
-    a.block = (int)ctx->trace_block;
-    a.stack = (int)ctx->trace_stack;
-    a.counts = nullptr;
-    a.scenes = nullptr;
-    a.offsets = nullptr;
-    a.num_scenes = 0;
     cudaError_t e = launch_trace(ctx->stream, a, any_hit);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "trace launch");
     return HCC_OK;
@@ -1198,27 +1342,11 @@ hcc_status hcc_trace_counts(hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *ra
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(static_cast<char *>(tmp.p) +
                                                                      rays->n * sizeof(hcc_hit));
     cudaError_t e = cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), ctx->stream);
-    TraceArgs a;
-    a.nodes = bvh->d_nodes;
-    a.layout = bvh->layout;
-    a.tris = bvh->d_tris;
-    a.root_ref = bvh->root_ref;
-    a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
-    a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
-    a.rs = ray_rs(rays);
-    a.rec = ray_rec(rays);
-    a.n = rays->n;
+    TraceArgs a = trace_args(ctx, bvh, rays, any_hit);
     a.gather = perm;
     a.scatter = perm;
     a.hits = reinterpret_cast<int4 *>(tmp.p);
-    a.err = ctx->d_err;
-    a.work = trace_work(ctx, any_hit);
-    a.block = (int)ctx->trace_block;
-    a.stack = (int)ctx->trace_stack;
     a.counts = cnt;
-    a.scenes = nullptr;
-    a.offsets = nullptr;
-    a.num_scenes = 0;
     if (e == cudaSuccess) e = launch_trace(ctx->stream, a, any_hit);
     unsigned long long host[4] = {0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, cnt, sizeof host, cudaMemcpyDeviceToHost, ctx->stream);
@@ -1246,6 +1374,7 @@ hcc_status hcc_batch_create(hcc_ctx *ctx, uint32_t num_scenes, const hcc_bvh *co
     }
     if (offsets[num_scenes] > HCC_MAX_SORT_N) return fail(ctx, HCC_ERR_INVALID_ARG, "batch above HCC_MAX_SORT_N rays");
     std::vector<hcc::SceneDesc> sd(num_scenes);
+    uint32_t compact_stack = 0;
     for (uint32_t s = 0; s < num_scenes; ++s) {
         const hcc_bvh *b = bvhs[s];
         hcc::SceneDesc &d = sd[s];
@@ -1255,6 +1384,10 @@ hcc_status hcc_batch_create(hcc_ctx *ctx, uint32_t num_scenes, const hcc_bvh *co
         d.prim_rec = b->d_prim_rec;
         d.root_ref = b->root_ref;
         d.num_tris = b->num_tris;
+        d.cnodes = b->d_compact;
+        d.croot = b->compact_root;
+        d.grid = b->grid;
+        compact_stack = std::max(compact_stack, b->compact_stack);
         const hcc_cut *c = cuts ? cuts[s] : nullptr;
         d.cut = c ? c->d_boxes : nullptr;
         d.used = c ? c->on_device : 0;
@@ -1272,6 +1405,7 @@ hcc_status hcc_batch_create(hcc_ctx *ctx, uint32_t num_scenes, const hcc_bvh *co
     bt->device = ctx->device;
     bt->layout = bvhs[0]->layout;
     bt->num_scenes = num_scenes;
+    bt->compact_stack = compact_stack;
     while ((1u << bt->scene_bits) < num_scenes) ++bt->scene_bits;
     bt->offsets.assign(offsets, offsets + num_scenes + 1);
     DeviceGuard g(ctx->device);
@@ -1321,6 +1455,7 @@ hcc_status hcc_batch_run(hcc_ctx *ctx, const hcc_batch *b, hcc_method method, co
     DeviceGuard g(ctx->device);
     TraceArgs a;
     a.layout = b->layout;
+    a.cstack = b->compact_stack;
     a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
     a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
     a.rs = ray_rs(rays);

@@ -37,6 +37,27 @@ constexpr uint32_t REF_TRI_MASK = 0x1FFFFFFFu;
 // child: lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, references, zeros; an unused
 // child has ref 0xFFFFFFFF.  An internal reference indexes wide nodes.
 
+// Compact layout (what traces walk; the layouts above are walked where it does
+// not apply): one 4-ary node = 64 bytes = four uint4.  Words 3c..3c+2 hold
+// child c's slab on each axis as two 16-bit bounds, lo in the low half and hi
+// in the high half; words 12..15 are the references (as above, an internal
+// one indexing compact nodes).  A bound q stands for the float with bits
+// 0x40000000 | q << 8, a coordinate of the scene's grid in [2, 8):
+// M(x) = (x - grid.lo) * grid.scale + GRID_ORIGIN per axis.  Bounds are rounded
+// outward with GRID_MARGIN to spare.  An unused child has lo = 0xFFFF above
+// hi = 0 on every axis, which no ray meets, and reference 0xFFFFFFFF.
+constexpr float GRID_ORIGIN = 2.0009765625f;     // 2 + 2^-10
+constexpr float GRID_SPAN = 5.9921875f;          // 6 - 2^-7: M(hi) stays below 8 - 2^-8
+constexpr float GRID_MARGIN = 3.147125244e-05f;  // 2^-15 + 2^-20, half the grid's smallest step
+// A ray whose origin lies further than this from the grid's zero is traced
+// from the point where it enters the scene: within it, the rounding of the
+// ray's grid coordinates and of its slab distances stays below GRID_MARGIN.
+constexpr float GRID_REACH = 32.0f;
+
+struct Grid {
+    float lo[3], scale[3];
+};
+
 // Triangle record = three float4: (v0.xyz, id bits), (e1.xyz, 0), (e2.xyz, 0)
 // with e1 = v1 - v0, e2 = v2 - v0 rounded to float.
 
@@ -53,6 +74,9 @@ struct SceneDesc {
     float lo[3], ext[3], L;
     uint32_t num_tris;
     uint32_t cut_ordered;  // every cut box has lo <= hi on every axis
+    const uint4 *cnodes;   // compact nodes (NULL: none), their root reference and grid
+    uint32_t croot;
+    Grid grid;
 };
 
 // Scene of ray src in a batch: the last s with offsets[s] <= src.
@@ -147,6 +171,10 @@ struct TraceArgs {
     int layout = 0;          // 0 = 32-byte quantised, 1 = 64-byte exact, 2 = 128-byte wide
     const float4 *tris = nullptr;  // 3 per triangle
     uint32_t root_ref = 0;
+    const uint4 *cnodes = nullptr;  // compact nodes, their root and grid (batches: in the scene table) ...
+    uint32_t croot = 0;
+    Grid grid = {};
+    uint32_t cstack = 0xFFFFFFFFu;  // ... and the stack entries a walk of them may need; walked where they suffice
     const float4 *org = nullptr;
     const float4 *dir = nullptr;
     uint32_t rs = 1;     // ray i is org/dir[i * rs]

@@ -30,7 +30,7 @@
 
 namespace hcc {
 // Device views of the opaque handles (hcc_api.cu).
-void bvh_view(const hcc_bvh *b, SceneDesc *out, int *layout, int *device);
+void bvh_view(const hcc_bvh *b, SceneDesc *out, int *layout, uint32_t *compact_stack, int *device);
 void cut_view(const hcc_cut *c, const float4 **boxes, uint32_t *on_device, int *device);
 }  // namespace hcc
 
@@ -70,6 +70,7 @@ struct hcc_server {
     std::vector<hcc::SceneDesc> scenes;
     std::vector<const float4 *> cut_boxes;
     std::vector<uint32_t> cut_used;
+    std::vector<uint32_t> compact_stack;  // per scene: stack entries its compact nodes fit in
     std::vector<Slot> slots;
     cudaMemPool_t pool = nullptr;
 
@@ -138,6 +139,10 @@ hcc_status launch_request(hcc_server *s, const Request &r, Slot &sl) {
     a.layout = s->layout;
     a.tris = sc.tris;
     a.root_ref = sc.root_ref;
+    a.cnodes = sc.cnodes;
+    a.croot = sc.croot;
+    a.grid = sc.grid;
+    a.cstack = s->compact_stack[r.scene];
     a.org = org;
     a.dir = dir;
     a.n = n;
@@ -291,11 +296,12 @@ hcc_status hcc_server_create(int device, uint32_t num_scenes, const hcc_bvh *con
     s->scenes.resize(num_scenes);
     s->cut_boxes.assign(num_scenes, nullptr);
     s->cut_used.assign(num_scenes, 0);
+    s->compact_stack.assign(num_scenes, 0xFFFFFFFFu);
     for (uint32_t k = 0; k < num_scenes; ++k) {
         int layout = 0, dev = 0;
         bool ok = bvhs[k] != nullptr;
         if (ok) {
-            hcc::bvh_view(bvhs[k], &s->scenes[k], &layout, &dev);
+            hcc::bvh_view(bvhs[k], &s->scenes[k], &layout, &s->compact_stack[k], &dev);
             if (k == 0) s->layout = layout;
             ok = layout == s->layout && dev == device;
         }

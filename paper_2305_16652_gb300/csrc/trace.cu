@@ -4,12 +4,15 @@
 // internal node holding its children's boxes (32-byte 8-bit quantised
 // layout or 64-byte exact FP32 layout of the BVH2, or 128-byte 4-ary nodes
 // collapsed from it), a per-thread stack of (node, entry distance) pairs.
+// Every layout's traces walk the compact 64-byte 4-ary nodes instead where the
+// scene and the stack allow it (launch_layout); the layout's own nodes serve the
+// other scenes and the counting diagnostic.
 //
 // Robustness: decoded child boxes are rounded outward (they contain the exact
 // boxes), the far slab distance is widened by 1 + 2*gamma(3) to cover the
 // rounding of the distances (Ize 2013, "Robust BVH Ray Traversal"; the wide
 // nodes' directed-rounding distances leave only the reciprocal's rounding
-// to cover), and a subtree is dropped only when its entry
+// to cover, the compact nodes' bounds hold a margin for it), and a subtree is dropped only when its entry
 // distance exceeds the best hit by more than 2^-16 relative, so traversal
 // never loses a triangle that the closest-hit definition would pick.
 // Triangle arithmetic is the canonical Moller-Trumbore sequence with explicit
@@ -18,6 +21,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -35,12 +39,17 @@ constexpr float PRUNE_SLACK = 1.0f + 1.0f / 65536.0f;
 // order (rays fetched through a permutation), where waiting longer keeps the
 // warp's neighbouring rays together (measured faster for each)
 constexpr uint32_t REFILL_MIN = 12;
-// resident threads per SM the persistent kernel is built for: binary nodes
-// (48 registers at 128-thread blocks), and wide nodes or a batch of scenes
-// (56); the register cap follows from threads x registers <= 64K
-constexpr int POOL_THREADS = 1280;
-constexpr int POOL_THREADS_WIDE = 1152;
 constexpr uint32_t REFILL_MIN_SORTED = 24;
+// ... and over compact nodes in either order: there a round is run by the whole
+// warp and costs little, so lanes need not wait as long (room's 16.6M rays in HCC
+// order, whole bounce: 3.97 ms at 8, 4.00 at 4 and 12, 4.20 at 24)
+constexpr uint32_t REFILL_MIN_COMPACT = 8;
+// resident threads per SM the persistent kernel is built for; the register cap
+// follows from threads x registers <= 64K: exact and quantised binary nodes
+// (48 registers at 128-thread blocks), wide nodes or a batch of scenes (56), and
+// compact nodes (64; at 56 or 48 registers the loop spills and more warps share
+// the L1: 4.06 against 3.97 ms for the bounce above at 56, 72 registers 4.11)
+constexpr int pool_threads(int layout, bool multi) { return layout == 3 ? 1024 : layout == 2 || multi ? 1152 : 1280; }
 
 __device__ __forceinline__ float byte_to_float(uint32_t w, uint32_t sel) {
     // 0x4B0000bb as float is 2^23 + bb exactly
@@ -84,31 +93,30 @@ __device__ __forceinline__ void slab(const Ray &r, const Box2 &b, float tcap, fl
     tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
 }
 
-// Moller-Trumbore on record k; returns true with (t, u, v) on a hit in
-// (tmin, tmax).  Same operation sequence as the definition: p = d x e2,
+// Moller-Trumbore; returns true with (t, u, v) if the ray's line meets the
+// triangle (the caller checks t against the ray's interval).  Same operation sequence as the definition: p = d x e2,
 // det = e1 . p, s = o - v0, u = (s . p) / det, q = s x e1, v = (d . q) / det,
 // t = (e2 . q) / det; dot(a, b) = fma(az, bz, fma(ay, by, ax * bx)),
 // cross(a, b).x = fma(ay, bz, -(az * by)) and cyclically.
-__device__ __forceinline__ bool intersect(const Ray &r, const float4 &A, const float4 &E1, const float4 &E2, float &t,
-                                          float &u, float &v) {
-    const float px = __fmaf_rn(r.dy, E2.z, -__fmul_rn(r.dz, E2.y));
-    const float py = __fmaf_rn(r.dz, E2.x, -__fmul_rn(r.dx, E2.z));
-    const float pz = __fmaf_rn(r.dx, E2.y, -__fmul_rn(r.dy, E2.x));
+__device__ __forceinline__ bool intersect(float ox, float oy, float oz, float dx, float dy, float dz, const float4 &A,
+                                          const float4 &E1, const float4 &E2, float &t, float &u, float &v) {
+    const float px = __fmaf_rn(dy, E2.z, -__fmul_rn(dz, E2.y));
+    const float py = __fmaf_rn(dz, E2.x, -__fmul_rn(dx, E2.z));
+    const float pz = __fmaf_rn(dx, E2.y, -__fmul_rn(dy, E2.x));
     const float det = __fmaf_rn(E1.z, pz, __fmaf_rn(E1.y, py, __fmul_rn(E1.x, px)));
-    if (det == 0.0f) return false;
     const float inv = __frcp_rn(det);
-    const float sx = __fsub_rn(-r.nxy.x, A.x), sy = __fsub_rn(-r.nxy.y, A.y), sz = __fsub_rn(-r.nzz.x, A.z);
+    const float sx = __fsub_rn(ox, A.x), sy = __fsub_rn(oy, A.y), sz = __fsub_rn(oz, A.z);
     u = __fmul_rn(__fmaf_rn(sz, pz, __fmaf_rn(sy, py, __fmul_rn(sx, px))), inv);
-    if (u < 0.0f || u > 1.0f) return false;
     const float qx = __fmaf_rn(sy, E1.z, -__fmul_rn(sz, E1.y));
     const float qy = __fmaf_rn(sz, E1.x, -__fmul_rn(sx, E1.z));
     const float qz = __fmaf_rn(sx, E1.y, -__fmul_rn(sy, E1.x));
-    v = __fmul_rn(__fmaf_rn(r.dz, qz, __fmaf_rn(r.dy, qy, __fmul_rn(r.dx, qx))), inv);
-    if (v < 0.0f || __fadd_rn(u, v) > 1.0f) return false;
+    v = __fmul_rn(__fmaf_rn(dz, qz, __fmaf_rn(dy, qy, __fmul_rn(dx, qx))), inv);
     t = __fmul_rn(__fmaf_rn(E2.z, qz, __fmaf_rn(E2.y, qy, __fmul_rn(E2.x, qx))), inv);
-    return t > r.tmin && t < r.tmax;
+    // as !(x < 0): a NaN is not rejected here, and t is then NaN as well
+    return det != 0.0f && !(u < 0.0f) && !(u > 1.0f) && !(v < 0.0f) && !(__fadd_rn(u, v) > 1.0f);
 }
 
+constexpr int COMPACT = 3;  // kernel layout number of the compact nodes (0-2: hcc_bvh_layout)
 constexpr uint32_t REF_NONE = 0xFFFFFFFFu;  // no node (empty stack, no postponed leaf)
 
 // Both children's boxes of an internal node, decoded for the slab test.
@@ -275,10 +283,10 @@ __device__ __forceinline__ uint32_t ray_pop(RayState &s, const uint2 *stack) {
 constexpr int LEAF_SLACK = 3;
 constexpr int LEAF_MIN = 4;
 template <bool ANY>
-__device__ __forceinline__ bool leaves_ready(const RayState &s) {
-    if (ANY) return __all_sync(__activemask(), s.leaf != REF_NONE);
+__device__ __forceinline__ bool leaves_ready(uint32_t leaf) {
+    if (ANY) return __all_sync(__activemask(), leaf != REF_NONE);
     const uint32_t active = __activemask();
-    const uint32_t parked = __ballot_sync(active, s.leaf != REF_NONE);
+    const uint32_t parked = __ballot_sync(active, leaf != REF_NONE);
     return __popc(parked) + LEAF_SLACK >= __popc(active);
 }
 
@@ -337,7 +345,7 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
             s.leaf = s.node;
             s.node = ray_pop(s, stack);
         }
-        if (leaves_ready<ANY>(s)) break;
+        if (leaves_ready<ANY>(s.leaf)) break;
     }
     // internal nodes: descend until (nearly) every lane has a leaf parked
     while (LAYOUT != 2 && s.node != REF_NONE && !(s.node & REF_LEAF)) {
@@ -373,7 +381,7 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
             s.leaf = s.node;
             s.node = ray_pop(s, stack);
         }
-        if (leaves_ready<ANY>(s)) break;
+        if (leaves_ready<ANY>(s.leaf)) break;
     }
     // leaves: the parked one, then any leaf that is next on the stack
     while (s.leaf != REF_NONE) {
@@ -385,7 +393,8 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
             const float4 A = __ldg(rec), E1 = __ldg(rec + 1), E2 = __ldg(rec + 2);
             if (COUNT) ++cn.tris;
             float t, u, v;
-            if (!intersect(s.r, A, E1, E2, t, u, v)) continue;
+            if (!intersect(-s.r.nxy.x, -s.r.nxy.y, -s.r.nzz.x, s.r.dx, s.r.dy, s.r.dz, A, E1, E2, t, u, v)) continue;
+            if (!(t > s.r.tmin && t < s.r.tmax)) continue;
             const int32_t prim = __float_as_int(A.w);
             if (s.best_prim < 0 || t < s.best_t || (t == s.best_t && prim < s.best_prim)) {
                 s.best_t = t;
@@ -412,9 +421,326 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
     }
 }
 
+// ---------------------------------------------------------------- compact nodes
+//
+// Why these nodes: a trace over the exact binary nodes kept the L1 data pipe 72 %
+// busy (two 32-byte loads per lane and visit, each lane its own line; the wide
+// nodes, seven 16-byte loads, 85 %) and waited for loads in 7.6 of 16 cycles per
+// instruction.  A compact node is read with two 32-byte loads for four children, so a
+// ray needs 16 visits and 33 loads where the binary nodes take 36 and 72, and the room's
+// nodes shrink from 32 to 13 MB.  What bounds the walk now (ncu, 0.96M rays): the
+// ALU pipe 71 %, issue 61 %, L1 data pipe 58 % busy, waits for loads 4.3 of 11.5
+// cycles per instruction; 154M warp instructions against 212M.
+
+// Traversal state over compact 4-ary nodes.  The slab test works in the
+// scene's grid: per axis tau = b * inv + c with b a decoded bound, inv the
+// reciprocal of the grid-space direction and c = -(origin * inv), one fma per
+// bound.  Its rounding, and that of the ray's grid coordinates, is below the
+// margin by which the stored bounds were widened, so no factor on the far
+// distance is needed.  tau is the ray's parameter t measured from `from` (tmin, or
+// the entry into the scene for an origin far outside it) and scaled by a power
+// of two that brings the scene's far side below 1: a saturating fma then
+// clamps the entry distance to the ray's start.
+struct CompactState {
+    float2 ixy, cxy;
+    float iz, cz;
+    uint32_t sx, sy, sz;  // byte selectors of each axis's near bound (lo or hi by the direction's sign)
+    float tcap;           // tau of the best hit widened by the prune slack
+    float widen;          // added to a box's exit distance (0 unless the origin is far outside the scene)
+    float ox, oy, oz, dx, dy, dz;
+    float best_t, best_u, best_v;
+    int32_t best_prim;
+    uint32_t sp;          // local address of the next free stack entry
+    uint32_t node, leaf;  // subtree to descend and parked leaf, or REF_NONE
+    uint32_t top_ref;     // copy of the topmost stack entry
+    float top_t;
+    static constexpr bool overflow = false;  // launch_trace walks compact nodes only where the stack suffices
+};
+
+// Stack slots below the pending subtrees: (tmin, scale) and (from, -), read only when a triangle is met.
+constexpr int COMPACT_SLOTS = 2;
+// relative widening of the exit distance of rays from far outside the scene:
+// the triangle test's own rounding grows with the distance to the origin, as
+// the widening of the other layouts' slab test (ROBUST_FAR) does
+constexpr float FAR_WIDEN = 1.0f / 1048576.0f;
+// ... and its limit, below the gap between the bounds of an unused child: 5.99
+// grid units on the axis that leaves the scene first, whose far side lies at
+// most GRID_REACH + 8 units from the start and at tau 1/4 or more
+constexpr float FAR_WIDEN_MAX = 1.0f / 32.0f;
+constexpr uint32_t GRID_HI_LO = 0x0220u;  // turns the selector of one bound of a word into the other's
+
+// A 16-bit bound of word w as a grid coordinate in [2, 8): bytes (0, low, high, 0x40).
+__device__ __forceinline__ float grid_bound(uint32_t w, uint32_t sel) {
+    return __uint_as_float(__byte_perm(w, 0x40u, sel));
+}
+
+// A ray whose origin is more than GRID_REACH from the grid's zero: measures t
+// from the point where it enters the scene's neighbourhood (one unit around the
+// grid's box), computed in double, so that the grid coordinates of the slab test
+// stay small.  Returns false if it never comes near.
+__device__ __noinline__ bool enter_grid(const float4 o4, const float4 d4, const Grid &g, float3 &p, float &from) {
+    const float o[3] = {o4.x, o4.y, o4.z}, d[3] = {d4.x, d4.y, d4.z};
+    double op[3], dp[3], tin = (double)o4.w, tout = (double)d4.w;
+    for (int k = 0; k < 3; ++k) {
+        op[k] = ((double)o[k] - (double)g.lo[k]) * (double)g.scale[k] + (double)GRID_ORIGIN;
+        dp[k] = (double)d[k] * (double)g.scale[k];
+        if (dp[k] == 0.0) {
+            if (!(op[k] >= 1.0 && op[k] <= 9.0)) return false;
+        } else {
+            const double a = (1.0 - op[k]) / dp[k], b = (9.0 - op[k]) / dp[k];
+            tin = fmax(tin, fmin(a, b));
+            tout = fmin(tout, fmax(a, b));
+        }
+    }
+    if (!(tin <= tout)) return false;
+    from = __double2float_rd(tin);
+    p.x = (float)(op[0] + (double)from * dp[0]);
+    p.y = (float)(op[1] + (double)from * dp[1]);
+    p.z = (float)(op[2] + (double)from * dp[2]);
+    // beyond about 10^8 scene sizes `from` no longer resolves the scene
+    return fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)) <= GRID_REACH;
+}
+
+__device__ __forceinline__ uint32_t local_address(const void *p) {
+    uint64_t a;
+    asm("cvta.to.local.u64 %0, %1;" : "=l"(a) : "l"(p));
+    return (uint32_t)a;
+}
+
+// As safe_inv, for a grid-space direction.
+__device__ __forceinline__ float grid_inv(float d) {
+    return __frcp_rn(fabsf(d) > 1e-36f ? d : copysignf(1e-36f, d));
+}
+
+// A lane without a ray.
+__device__ __forceinline__ void ray_none(CompactState &s, uint32_t stack_base) {
+    s.node = s.leaf = REF_NONE;
+    s.sp = stack_base;
+}
+
+__device__ __forceinline__ bool ray_done(const CompactState &s, uint32_t stack_base) {
+    return s.node == REF_NONE && s.leaf == REF_NONE && s.sp == stack_base;
+}
+
+__device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const float4 o4, const float4 d4,
+                                         const Grid &g, uint32_t root) {
+    s.ox = o4.x;
+    s.oy = o4.y;
+    s.oz = o4.z;
+    s.dx = d4.x;
+    s.dy = d4.y;
+    s.dz = d4.z;
+    float3 p = make_float3(__fmaf_rn(__fsub_rn(o4.x, g.lo[0]), g.scale[0], GRID_ORIGIN),
+                           __fmaf_rn(__fsub_rn(o4.y, g.lo[1]), g.scale[1], GRID_ORIGIN),
+                           __fmaf_rn(__fsub_rn(o4.z, g.lo[2]), g.scale[2], GRID_ORIGIN));
+    const float ix = grid_inv(__fmul_rn(d4.x, g.scale[0])), iy = grid_inv(__fmul_rn(d4.y, g.scale[1])),
+                iz = grid_inv(__fmul_rn(d4.z, g.scale[2]));
+    float from = o4.w, start = o4.w;  // start: `from` as seen from p
+    const bool far = fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)) > GRID_REACH;
+    bool meets = true;
+    if (far) {
+        meets = enter_grid(o4, d4, g, p, from);
+        start = 0.0f;
+    }
+    // c, and the far side of the scene, in t from `from`
+    const float cx = __fmaf_rn(-p.x, ix, -start), cy = __fmaf_rn(-p.y, iy, -start), cz = __fmaf_rn(-p.z, iz, -start);
+    const float leave = fmin3(__fmaf_rn(ix < 0.0f ? 2.0f : 8.0f, ix, cx), __fmaf_rn(iy < 0.0f ? 2.0f : 8.0f, iy, cy),
+                              __fmaf_rn(iz < 0.0f ? 2.0f : 8.0f, iz, cz));
+    const float tmax = __fsub_ru(d4.w, from);
+    // 2^-(e + 2) for a far side in [2^e, 2^(e+1)); a far side at or before the start is a miss
+    const uint32_t e = __float_as_uint(fmaxf(leave, 2e-38f)) >> 23;
+    const float scale = __uint_as_float((252u - (e < 251u ? e : 251u)) << 23);
+    meets = meets && leave > 0.0f && tmax > 0.0f;
+    s.ixy = make_float2(__fmul_rn(ix, scale), __fmul_rn(iy, scale));
+    s.iz = __fmul_rn(iz, scale);
+    s.cxy = make_float2(__fmul_rn(cx, scale), __fmul_rn(cy, scale));
+    s.cz = __fmul_rn(cz, scale);
+    s.sx = ix < 0.0f ? 0x4325u : 0x4105u;
+    s.sy = iy < 0.0f ? 0x4325u : 0x4105u;
+    s.sz = iz < 0.0f ? 0x4325u : 0x4105u;
+    s.tcap = __fmul_ru(tmax, scale);
+    s.widen = far ? fminf(__fmul_rn(__fmul_rn(fabsf(from), FAR_WIDEN), scale), FAR_WIDEN_MAX) : 0.0f;
+    s.best_t = d4.w;
+    s.best_u = s.best_v = 0.0f;
+    s.best_prim = -1;
+    stack[0] = make_uint2(__float_as_uint(o4.w), __float_as_uint(scale));
+    stack[1] = make_uint2(__float_as_uint(from), 0u);
+    s.node = meets ? root : REF_NONE;
+    s.leaf = REF_NONE;
+}
+
+// A leaf that is next becomes the lane's parked leaf if it has none (a node of
+// REF_NONE changes nothing).  Predicated moves: no branch, and off the ALU pipe.
+__device__ __forceinline__ void park_leaf(CompactState &s) {
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.eq.u32 p, %1, 0xffffffff;\n\t"
+        "setp.lt.and.s32 p, %0, 0, p;\n\t"
+        "@p mov.b32 %1, %0;\n\t"
+        "@p mov.b32 %0, 0xffffffff;\n\t}"
+        : "+r"(s.node), "+r"(s.leaf));
+}
+
+// Takes the next pending subtree if the lane has none to descend; one beyond
+// the best hit is dropped (the lane tries again in the next step).  The topmost
+// entry is kept in registers and its successor is loaded when it is taken, so a
+// pop does not wait for local memory.  (Any hit: the best hit never moves, so
+// entries are references only.)
+template <bool ANY>
+__device__ __forceinline__ void pop_node(CompactState &s, uint32_t stack_base) {
+    if (ANY) {
+        asm volatile("{\n\t.reg .pred p;\n\t"
+            "setp.eq.u32 p, %0, 0xffffffff;\n\t"
+            "setp.ne.and.u32 p, %1, %2, p;\n\t"
+            "@p add.u32 %1, %1, -4;\n\t"
+            "@p ld.local.b32 %0, [%1];\n\t}"
+            : "+r"(s.node), "+r"(s.sp) : "r"(stack_base) : "memory");
+        return;
+    }
+    asm volatile("{\n\t.reg .pred p, q;\n\t"
+        "setp.eq.u32 p, %0, 0xffffffff;\n\t"
+        "setp.ne.and.u32 p, %1, %5, p;\n\t"
+        "setp.le.and.f32 q, %3, %4, p;\n\t"
+        "@q mov.b32 %0, %2;\n\t"
+        "@p add.u32 %1, %1, -8;\n\t"
+        "@p ld.local.v2.b32 {%2, %3}, [%1+-8];\n\t}"
+        : "+r"(s.node), "+r"(s.sp), "+r"(s.top_ref), "+f"(s.top_t) : "f"(s.tcap), "r"(stack_base) : "memory");
+}
+
+// Entry and exit distance of a child (slab words wx, wy, wz).  The near and far
+// bound of an axis come out of its word by byte permutes whose selectors hold the
+// direction's sign, so decoding costs no more than sorting the two distances by
+// min and max would.
+__device__ __forceinline__ void compact_child(const CompactState &s, uint32_t wx, uint32_t wy, uint32_t wz, float &tn,
+                                              float &tf) {
+    const float2 n = __ffma2_rn(make_float2(grid_bound(wx, s.sx), grid_bound(wy, s.sy)), s.ixy, s.cxy);
+    const float2 f = __ffma2_rn(make_float2(grid_bound(wx, s.sx ^ GRID_HI_LO), grid_bound(wy, s.sy ^ GRID_HI_LO)),
+                                s.ixy, s.cxy);
+    const float nz = __saturatef(__fmaf_rn(grid_bound(wz, s.sz), s.iz, s.cz));
+    const float fz = __fmaf_rn(grid_bound(wz, s.sz ^ GRID_HI_LO), s.iz, s.cz);
+    tn = fmax3(n.x, n.y, nz);
+    tf = fminf(__fadd_rn(fmin3(f.x, f.y, fz), s.widen), s.tcap);
+}
+
+// Pushes a subtree met at distance t (+inf: not met).  TOP: the last push of a
+// step, which leaves the topmost entry.
+template <bool TOP>
+__device__ __forceinline__ void push_node(CompactState &s, uint32_t ref, float t) {
+    if (TOP)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %4, 0f7F800000;\n\t"
+            "@p st.local.v2.b32 [%0], {%3, %4};\n\t@p add.u32 %0, %0, 8;\n\t@p mov.b32 %1, %3;\n\t@p mov.b32 %2, %4;\n\t}"
+            : "+r"(s.sp), "+r"(s.top_ref), "+f"(s.top_t) : "r"(ref), "f"(t) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %2, 0f7F800000;\n\t"
+            "@p st.local.v2.b32 [%0], {%1, %2};\n\t@p add.u32 %0, %0, 8;\n\t}"
+            : "+r"(s.sp) : "r"(ref), "f"(t) : "memory");
+}
+
+// One node step: tests the four children, descends into the nearest one met
+// and pushes the others, farthest first.  (Pushing them unsorted saved 10
+// instructions of 185 a step but took 13 % more steps; multiply-adds in place of
+// the selects of the exchanges, to relieve the ALU pipe, changed nothing.)
+template <bool ANY>
+__device__ __forceinline__ void node_step(CompactState &s, const uint4 *__restrict__ nodes) {
+    uint4 w0, w1, w2, rf;
+    ldg256(nodes + 4 * (size_t)s.node, w0, w1);
+    ldg256(nodes + 4 * (size_t)s.node + 2, w2, rf);
+    float n0, n1, n2, n3, f0, f1, f2, f3;
+    compact_child(s, w0.x, w0.y, w0.z, n0, f0);
+    compact_child(s, w0.w, w1.x, w1.y, n1, f1);
+    compact_child(s, w1.z, w1.w, w2.x, n2, f2);
+    compact_child(s, w2.y, w2.z, w2.w, n3, f3);
+    if (ANY) {
+        // no order and no distance: every met child is pushed, the last taken back
+        asm volatile("{\n\t.reg .pred h0, h1, h2, h3, p;\n\t"
+            "setp.lt.f32 h0, %2, %6;\n\tsetp.lt.f32 h1, %3, %7;\n\tsetp.lt.f32 h2, %4, %8;\n\tsetp.lt.f32 h3, %5, %9;\n\t"
+            "mov.b32 %0, 0xffffffff;\n\t"
+            "@h0 st.local.b32 [%1], %10;\n\t@h0 add.u32 %1, %1, 4;\n\t@h0 mov.b32 %0, %10;\n\t"
+            "@h1 st.local.b32 [%1], %11;\n\t@h1 add.u32 %1, %1, 4;\n\t@h1 mov.b32 %0, %11;\n\t"
+            "@h2 st.local.b32 [%1], %12;\n\t@h2 add.u32 %1, %1, 4;\n\t@h2 mov.b32 %0, %12;\n\t"
+            "@h3 st.local.b32 [%1], %13;\n\t@h3 add.u32 %1, %1, 4;\n\t@h3 mov.b32 %0, %13;\n\t"
+            "setp.ne.u32 p, %0, 0xffffffff;\n\t@p add.u32 %1, %1, -4;\n\t}"
+            : "=&r"(s.node), "+r"(s.sp)
+            : "f"(n0), "f"(n1), "f"(n2), "f"(n3), "f"(f0), "f"(f1), "f"(f2), "f"(f3), "r"(rf.x), "r"(rf.y), "r"(rf.z), "r"(rf.w)
+            : "memory");
+        return;
+    }
+    const float INF = __int_as_float(0x7F800000);
+    n0 = n0 < f0 ? n0 : INF;
+    n1 = n1 < f1 ? n1 : INF;
+    n2 = n2 < f2 ? n2 : INF;
+    n3 = n3 < f3 ? n3 : INF;
+    uint32_t r0 = rf.x, r1 = rf.y, r2 = rf.z, r3 = rf.w;
+    order2(n0, r0, n1, r1);
+    order2(n2, r2, n3, r3);
+    order2(n0, r0, n2, r2);
+    order2(n1, r1, n3, r3);
+    order2(n1, r1, n2, r2);
+    s.node = n0 < INF ? r0 : REF_NONE;
+    push_node<false>(s, r3, n3);
+    push_node<false>(s, r2, n2);
+    push_node<true>(s, r1, n1);
+}
+
+// One round over compact nodes, run by the whole warp together (a lane without
+// a ray takes part in the votes only): node steps until all but COMPACT_SLACK of
+// the lanes that could go on hold a parked leaf, then triangle tests, one triangle
+// per lane and step, while at least COMPACT_TRI_MIN lanes have one; a leaf that
+// is not finished stays parked for the next round.  A step keeps its branches
+// few (predicated pushes, pops and moves, all of the triangle test computed at
+// once): with a branch around each, a warp spent 30 of 206 instructions per node
+// step on branching, and pops alone in loops at 10 % of its lanes.  (The plain
+// rules for any hit, as for the other layouts: 592 us for 4.1M shadow rays and
+// their order against 596 with a slack of 4 lanes.)
+constexpr int COMPACT_SLACK = 6;    // 3: 1.5 % slower in HCC order, 5 % unsorted; 10: equal
+constexpr int COMPACT_TRI_MIN = 6;  // 4 and 8 within 0.5 %
+template <bool ANY>
+__device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, uint32_t stack_base,
+                                          const uint4 *__restrict__ nodes, const float4 *__restrict__ tris) {
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    bool more;
+    do {
+        pop_node<ANY>(s, stack_base);
+        park_leaf(s);
+        if ((int)s.node >= 0) node_step<ANY>(s, nodes);
+        park_leaf(s);
+        more = s.leaf == REF_NONE && (s.node != REF_NONE || s.sp != stack_base);
+    } while (__popc(__ballot_sync(FULL, more)) > (ANY ? 0 : COMPACT_SLACK));
+    while (__any_sync(FULL, s.leaf != REF_NONE)) {
+        if (s.leaf != REF_NONE) {
+            const float4 *rec = tris + 3 * (size_t)(s.leaf & REF_TRI_MASK);
+            const float4 A = __ldg(rec), E1 = __ldg(rec + 1), E2 = __ldg(rec + 2);
+            // the next triangle of the leaf, or the next leaf
+            if (s.leaf & ~(REF_LEAF | REF_TRI_MASK)) {
+                s.leaf -= REF_TRI_MASK;
+            } else {
+                s.leaf = REF_NONE;
+                park_leaf(s);
+            }
+            float t, u, v;
+            const bool met = intersect(s.ox, s.oy, s.oz, s.dx, s.dy, s.dz, A, E1, E2, t, u, v);
+            const int32_t prim = __float_as_int(A.w);
+            if (met && (t < s.best_t || (t == s.best_t && prim < s.best_prim))) {
+                const uint2 e0 = stack[0], e1 = stack[1];
+                if (t > __uint_as_float(e0.x)) {
+                    s.best_t = t;
+                    s.best_u = u;
+                    s.best_v = v;
+                    s.best_prim = prim;
+                    const float tau = __fsub_ru(t, __uint_as_float(e1.x));
+                    s.tcap = __fmul_ru(__fmaf_ru(__fadd_ru(fabsf(t), tau), PRUNE_SLACK - 1.0f, tau),
+                                       __uint_as_float(e0.y));
+                    if (ANY) ray_none(s, stack_base);
+                }
+            }
+        }
+        if (__popc(__ballot_sync(FULL, s.leaf != REF_NONE)) < (ANY ? 1 : COMPACT_TRI_MIN)) break;
+    }
+}
+
 // The hit record {prim, t, u, v} (prim -1 and t = +inf on a miss or a
 // stack overflow).
-__device__ __forceinline__ int4 ray_result(const RayState &s) {
+template <typename State>
+__device__ __forceinline__ int4 ray_result(const State &s) {
     const bool miss = s.overflow || s.best_prim < 0;
     int4 out;
     out.x = miss ? -1 : s.best_prim;
@@ -434,11 +760,12 @@ __device__ __forceinline__ void add_counts(const TraceArgs &a, const Counters &c
     }
 }
 
-// Reads ray slot i: the ray is org/dir[gather[i]] (or i).  Returns false
-// (and reports) for an out-of-range permutation entry.
-template <bool MULTI>
-__device__ __forceinline__ bool fetch_ray(const TraceArgs &a, uint64_t i, float4 &o4, float4 &d4,
-                                          const uint4 *&nodes, const float4 *&tris, uint32_t &root) {
+// Reads ray slot i (the ray is org/dir[gather[i]], or i) and sets up its
+// traversal.  Returns false (and reports) for an out-of-range permutation entry.
+template <bool MULTI, int LAYOUT, typename State>
+__device__ __forceinline__ bool start_ray(const TraceArgs &a, uint64_t i, State &s, uint2 *stack,
+                                          const uint4 *&nodes, const float4 *&tris) {
+    float4 o4, d4;
     uint64_t src = i;
     if (a.gather) {
         src = a.gather[i];
@@ -455,20 +782,27 @@ __device__ __forceinline__ bool fetch_ray(const TraceArgs &a, uint64_t i, float4
         o4 = __ldcs(a.org + src * a.rs);
         d4 = __ldcs(a.dir + src * a.rs);
     }
-    nodes = a.nodes;
-    tris = a.tris;
-    root = a.root_ref;
-    if (MULTI) {
-        const SceneDesc &sc = a.scenes[scene_of(a.offsets, a.num_scenes, src)];
-        nodes = sc.nodes;
-        tris = sc.tris;
-        root = sc.root_ref;
+    const SceneDesc *sc = MULTI ? a.scenes + scene_of(a.offsets, a.num_scenes, src) : nullptr;
+    tris = MULTI ? sc->tris : a.tris;
+    if constexpr (LAYOUT == COMPACT) {
+        nodes = MULTI ? sc->cnodes : a.cnodes;
+        ray_init(s, stack, o4, d4, MULTI ? sc->grid : a.grid, MULTI ? sc->croot : a.croot);
+    } else {
+        nodes = MULTI ? sc->nodes : a.nodes;
+        ray_init(s, o4, d4, MULTI ? sc->root_ref : a.root_ref);
     }
     return true;
 }
 
+template <int LAYOUT>
+using StateOf = std::conditional_t<LAYOUT == COMPACT, CompactState, RayState>;
+// Stack entries of a kernel with STACKN entries for pending subtrees.
+template <int LAYOUT, int STACKN>
+constexpr int STACK_SIZE = STACKN + (LAYOUT == COMPACT ? COMPACT_SLOTS : 0);
+
 // Writes the record of ray slot i to hits[scatter[i]] (or i).
-__device__ __forceinline__ void store_hit(const TraceArgs &a, uint64_t i, const RayState &s) {
+template <typename State>
+__device__ __forceinline__ void store_hit(const TraceArgs &a, uint64_t i, const State &s) {
     if (i >= a.n) {  // not a ray slot: report, never index the permutation out of bounds
         atomicOr(a.err, ERR_INDEX);
         return;
@@ -487,18 +821,26 @@ __device__ __forceinline__ void store_hit(const TraceArgs &a, uint64_t i, const 
 template <bool ANY, bool COUNT, int LAYOUT, bool MULTI>
 __global__ void __launch_bounds__(TRACE_BLOCK) k_trace(TraceArgs a) {
     uint64_t i = (uint64_t)blockIdx.x * TRACE_BLOCK + threadIdx.x;
-    if (i >= a.n) return;
-    if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end (blocks start in index order)
-    float4 o4, d4;
     const uint4 *nodes;
     const float4 *tris;
-    uint32_t root;
-    if (!fetch_ray<MULTI>(a, i, o4, d4, nodes, tris, root)) return;
-    RayState s;
-    uint2 stack[STACK];
+    StateOf<LAYOUT> s;
+    uint2 stack[STACK_SIZE<LAYOUT, STACK>];
     Counters cn;
-    ray_init(s, o4, d4, root);
-    while (!ray_done(s)) ray_round<ANY, COUNT, LAYOUT, STACK>(s, stack, nodes, tris, cn);
+    bool have = i < a.n;
+    if (have) {
+        if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end (blocks start in index order)
+        have = start_ray<MULTI, LAYOUT>(a, i, s, stack, nodes, tris);
+    }
+    if constexpr (LAYOUT == COMPACT) {
+        const uint32_t base = local_address(stack + COMPACT_SLOTS);
+        s.sp = base;
+        if (!have) ray_none(s, base);
+        while (__any_sync(0xFFFFFFFFu, !ray_done(s, base))) ray_round<ANY>(s, stack, base, nodes, tris);
+        if (!have) return;
+    } else {
+        if (!have) return;
+        while (!ray_done(s)) ray_round<ANY, COUNT, LAYOUT, STACK>(s, stack, nodes, tris, cn);
+    }
     store_hit(a, i, s);
     add_counts<COUNT>(a, cn);
 }
@@ -523,20 +865,22 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace(TraceArgs a) {
 // BLOCK threads per block and STACKN stack entries per ray are a shape the
 // autotuner may pick.
 template <bool ANY, bool COUNT, int LAYOUT, bool MULTI, int BLOCK, int STACKN>
-__global__ void __launch_bounds__(BLOCK, ((LAYOUT == 2 || MULTI) ? POOL_THREADS_WIDE : POOL_THREADS) / BLOCK)
+__global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
     k_trace_pool(TraceArgs a) {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     const uint32_t lane = threadIdx.x & 31;
     uint32_t lt;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
-    RayState s;
-    uint2 stack[STACKN];
+    StateOf<LAYOUT> s;
+    uint2 stack[STACK_SIZE<LAYOUT, STACKN>];
     Counters cn;
-    const uint4 *nodes = a.nodes;
-    const float4 *tris = a.tris;
-    uint64_t slot = 0;
+    const uint4 *nodes = nullptr;
+    const float4 *tris = nullptr;
+    uint32_t slot = 0;  // below n, which fits 32 bits
     bool have = false, exhausted = false;
-    const uint32_t refill_min = a.gather ? REFILL_MIN_SORTED : REFILL_MIN;
+    const uint32_t stack_base = LAYOUT == COMPACT ? local_address(stack + COMPACT_SLOTS) : 0u;
+    if constexpr (LAYOUT == COMPACT) ray_none(s, stack_base);
+    const uint32_t refill_min = LAYOUT == COMPACT ? REFILL_MIN_COMPACT : a.gather ? REFILL_MIN_SORTED : REFILL_MIN;
     for (;;) {
         const bool want = !have && !exhausted;
         const uint32_t need = __ballot_sync(FULL, want);
@@ -547,27 +891,30 @@ __global__ void __launch_bounds__(BLOCK, ((LAYOUT == 2 || MULTI) ? POOL_THREADS_
             if ((int)lane == leader) base = atomicAdd(a.work, (unsigned long long)__popc(need));
             base = __shfl_sync(FULL, base, leader);
             if (want) {
-                slot = base + __popc(need & lt);
-                if ((a.gather || a.scatter) && slot < a.n) slot = a.n - 1 - slot;  // sorted order from its end
-                if (slot < a.n) {
-                    float4 o4, d4;
-                    uint32_t root;
-                    if (fetch_ray<MULTI>(a, slot, o4, d4, nodes, tris, root)) {
-                        ray_init(s, o4, d4, root);
-                        have = true;
-                    }
+                const uint64_t at = base + __popc(need & lt);
+                if (at < a.n) {
+                    slot = (uint32_t)((a.gather || a.scatter) ? a.n - 1 - at : at);  // sorted order from its end
+                    have = start_ray<MULTI, LAYOUT>(a, slot, s, stack, nodes, tris);
                 } else {
                     exhausted = true;
                 }
             }
         }
         if (!__any_sync(FULL, have)) {
-            if (__all_sync(FULL, exhausted)) break;
+            if (__any_sync(FULL, exhausted)) break;
             continue;
         }
+        bool done;
+        if constexpr (LAYOUT == COMPACT) {
+            ray_round<ANY>(s, stack, stack_base, nodes, tris);
+            done = ray_done(s, stack_base);
+        }
         if (have) {
-            ray_round<ANY, COUNT, LAYOUT, STACKN>(s, stack, nodes, tris, cn);
-            if (ray_done(s)) {
+            if constexpr (LAYOUT != COMPACT) {
+                ray_round<ANY, COUNT, LAYOUT, STACKN>(s, stack, nodes, tris, cn);
+                done = ray_done(s);
+            }
+            if (done) {
                 store_hit(a, slot, s);
                 have = false;
             }
@@ -637,6 +984,19 @@ cudaError_t launch_pool_shaped(cudaStream_t s, const TraceArgs &a) {
 
 template <bool ANY, bool CNT, bool MULTI>
 cudaError_t launch_layout(cudaStream_t s, const TraceArgs &a, bool pool) {
+    // Compact nodes wherever they exist and their deepest stack fits the trace's.
+    // They replaced each layout's own nodes by measurement (whole call, own against
+    // compact): 16.6M rays in HCC order over exact nodes 4.75 -> 3.95 ms, 0.96M
+    // 420 -> 323 us, 2.1M unsorted over wide nodes 614 -> 438 us, 2M in TwoPoint
+    // order over quantised nodes 745 -> 557 us, 4.1M shadow rays 640 -> 599 us.
+    if constexpr (!CNT) {
+        const int depth = pool && !ANY ? a.stack : STACK;
+        if (a.cstack <= (uint32_t)depth) {
+            if (pool) return launch_pool_shaped<ANY, CNT, COMPACT, MULTI>(s, a);
+            k_trace<ANY, CNT, COMPACT, MULTI><<<(unsigned)((a.n + TRACE_BLOCK - 1) / TRACE_BLOCK), TRACE_BLOCK, 0, s>>>(a);
+            return cudaGetLastError();
+        }
+    }
     if (pool) {
         if (a.layout == 0) return launch_pool_shaped<ANY, CNT, 0, MULTI>(s, a);
         if (a.layout == 1) return launch_pool_shaped<ANY, CNT, 1, MULTI>(s, a);

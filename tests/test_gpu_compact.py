@@ -1,0 +1,102 @@
+"""The compact 4-ary nodes that traces walk (needs a GB300): closest hits equal the
+brute-force definition (oracle.trace_brute) where the grid's arithmetic is at its
+limits, and the other layouts' nodes take over where it does not apply."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2305_16652_gb300 import gen, hcc
+from parity import compare_hits
+from test_gpu_layouts import _rays, _trace
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = hcc.hcc_create(0)
+    yield c
+    hcc.hcc_destroy(c)
+
+
+def _check(ctx, tris, org, dir_, layout="exact"):
+    bvh = gen.build_bvh(tris)
+    h = hcc.hcc_bvh_upload(ctx, bvh, layout=layout)
+    try:
+        ref = oracle.trace_brute(tris, org, dir_)
+        compare_hits(_trace(ctx, h, org, dir_), ref)
+        occl = _trace(ctx, h, org, dir_, any_hit=True)["prim"] >= 0
+        assert np.array_equal(occl, ref["prim"] >= 0)
+        return ref
+    finally:
+        hcc.hcc_bvh_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1000, 38912, 155649, 160000])
+def test_partial_warps_and_first_refills(ctx, n):
+    """Wavefronts that end inside a warp, and around the first slots taken by refilling."""
+    tris = gen.random_tris(3, 60, mu=-1.5)
+    org, dir_ = _rays(n, n, tris)
+    _check(ctx, tris, org, dir_)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("distance", [0.0, 3.0, 6.0, 100.0])
+def test_axis_parallel_and_distant_rays(ctx, axis, distance):
+    """Directions with two zero components, from inside, within and beyond the grid's reach
+    (where a ray is measured from its entry into the scene)."""
+    tris = gen.random_tris(5, 400, mu=-1.5)
+    rng = np.random.default_rng(axis)
+    n = 1500
+    o = rng.random((n, 3))
+    d = np.zeros((n, 3))
+    d[:, axis] = np.where(rng.random(n) < 0.5, 1.0, -1.0)
+    if distance:
+        o[:, axis] = 0.5 - d[:, axis] * (distance + 0.5)
+    d[n // 2:] += rng.normal(scale=1e-3, size=(n - n // 2, 3))  # and nearly parallel ones
+    org = np.concatenate([o, np.full((n, 1), 1e-4)], 1).astype(np.float32)
+    dir_ = np.concatenate([d, np.full((n, 1), np.inf)], 1).astype(np.float32)
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 100
+
+
+@pytest.mark.parametrize("scale", [1e-6, 1.0, 1e5])
+def test_direction_and_scene_scales(ctx, scale):
+    tris = (gen.random_tris(9, 300, mu=-1.5) * np.float32(scale)).astype(np.float32)
+    org, dir_ = _rays(11, 2000, tris)
+    org[:, 3] = 0.0
+    dir_[:, :3] *= np.float32(37.0)  # not normalised
+    dir_[::3, 3] = np.float32(0.02 * scale)  # short intervals, and empty ones
+    dir_[1::7, 3] = 0.0
+    _check(ctx, tris, org, dir_)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_flat_scene(ctx, axis):
+    tris = gen.random_tris(13, 200, mu=-1.5).reshape(-1, 3, 3)
+    tris[:, :, axis] = 0.25
+    tris = np.ascontiguousarray(tris.reshape(-1, 9))
+    org, dir_ = _rays(17, 2000, tris)
+    org[: 200, axis] = 0.25  # rays in the plane itself
+    _check(ctx, tris, org, dir_)
+
+
+def test_negative_and_late_intervals(ctx):
+    tris = gen.random_tris(19, 400, mu=-1.5)
+    org, dir_ = _rays(23, 2000, tris)
+    org[:1000, 3] = -1.0
+    org[1000:, 3] = 0.7
+    _check(ctx, tris, org, dir_)
+
+
+@pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
+def test_scene_that_does_not_suit_the_grid(ctx, layout):
+    """Detail far below the grid's step (a cloud of 1e-6 units in a scene of 1): the layout's nodes are walked."""
+    small = (gen.random_tris(29, 300, mu=-1.5) * np.float32(1e-6)).astype(np.float32)
+    far = np.array([[0, 0, 1, 1, 0, 1, 0, 1, 1]], np.float32)
+    tris = np.ascontiguousarray(np.concatenate([small, far]))
+    org, dir_ = _rays(31, 2000, small)
+    org[:, 3] = 0.0
+    ref = _check(ctx, tris, org, dir_, layout)
+    assert (ref["prim"] >= 0).any()
