@@ -191,8 +191,8 @@ hcc_status hcc_set_twopoint_distance(hcc_ctx *ctx, float fraction);
 hcc_status hcc_set_sort_wait_limit(hcc_ctx *ctx, uint32_t status_reads);
 
 /* Test hook for the bounded wait above (no counterpart in the paper): while
- * set, tile number `tile` (3584 keys each) of every digit pass of this
- * context's sorts never publishes its counts, so the tile after it waits
+ * set, this context's sorts of any size run as digit passes over tiles of 3584
+ * keys and tile number `tile` of every pass never publishes its counts, so the tile after it waits
  * until its limit and the sort reports HCC_ERR_TIMEOUT.  0xFFFFFFFF (the
  * default) withholds nothing.  Never needed outside tests. */
 hcc_status hcc_test_sort_withhold_tile(hcc_ctx *ctx, uint32_t tile);
@@ -378,7 +378,8 @@ hcc_status hcc_key_stats(hcc_ctx *ctx, const void *keys, uint32_t key_bits, cons
  * orders ray indices).  perm[j] = id of the j-th ray in sorted order.
  * keys: n uint32_t (key_bits <= 32) or uint64_t (key_bits > 32), device,
  * not modified.  perm: n uint32_t, device, must not overlap keys.
- * LSD radix sort, 8-bit digits; digits that are equal for every key are
+ * LSD radix sort, 8-bit digits: up to 65,536 keys in one launch, above that
+ * one launch per digit, where digits that are equal for every key are
  * skipped, which leaves the result unchanged.  Scratch comes from the
  * context (see hcc_reserve).  n <= HCC_MAX_SORT_N.
  * Errors: INVALID_ARG, OOM, CUDA; TIMEOUT at hcc_sync if a bounded
