@@ -73,7 +73,6 @@ struct SceneDesc {
     uint32_t used;      // cut nodes that drive key bits
     float lo[3], ext[3], L;
     uint32_t num_tris;
-    uint32_t cut_ordered;  // every cut box has lo <= hi on every axis
     const uint4 *cnodes;   // compact nodes (NULL: none), their root reference and grid
     uint32_t croot;
     Grid grid;
