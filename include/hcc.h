@@ -146,7 +146,8 @@ hcc_status hcc_reserve(hcc_ctx *ctx, uint64_t max_n, uint32_t max_key_bits);
  * lanes of the warp are idle (24 when the rays are fetched through a sorted
  * permutation) (Aila & Laine 2009, "replacing terminated rays").  AUTO (the
  * default): REFILL for closest-hit traces, PER_RAY for any-hit traces
- * (measured faster for each on GB300).  Results do not depend
+ * (measured faster for each on GB300), and four threads per ray for
+ * single wavefronts of at most 80,000 rays, which do not fill the GPU.  Results do not depend
  * on the schedule, except which hit an any-hit query reports.
  */
 typedef enum hcc_trace_schedule {

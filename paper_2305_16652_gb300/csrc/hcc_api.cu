@@ -374,6 +374,7 @@ static TraceArgs trace_args(const hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_ra
     a.n = rays->n;
     a.err = ctx->d_err;
     a.work = trace_work(ctx, any_hit);
+    a.quads = ctx->schedule == HCC_TRACE_AUTO;
     a.block = (int)ctx->trace_block;
     a.stack = (int)ctx->trace_stack;
     return a;

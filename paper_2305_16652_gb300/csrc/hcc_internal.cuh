@@ -189,6 +189,7 @@ struct TraceArgs {
     const uint64_t *offsets = nullptr;     // scene s owns rays [offsets[s], offsets[s+1])
     uint32_t num_scenes = 0;
     unsigned long long *work = nullptr;    // slot counter of the persistent trace (NULL: one thread per slot)
+    bool quads = false;                    // small wavefronts may be traced with four lanes per ray
     int block = 128;                       // closest-hit persistent trace: threads per block ...
     int stack = HCC_TRACE_STACK;           // ... and stack entries per ray (a supported shape)
 };

@@ -148,6 +148,7 @@ hcc_status launch_request(hcc_server *s, const Request &r, Slot &sl) {
     a.n = n;
     a.hits = static_cast<int4 *>(d_hits);
     a.err = sl.d_err;
+    a.quads = true;
     // closest hit: persistent trace with ray replacement; any hit: one thread per ray
     a.work = r.any_hit ? nullptr : reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(sl.d_err) + 8);
     if (e == cudaSuccess && sorts) {

@@ -507,9 +507,11 @@ __device__ __forceinline__ uint32_t local_address(const void *p) {
     return (uint32_t)a;
 }
 
-// As safe_inv, for a grid-space direction.
+// As safe_inv, for a grid-space direction; one ulp of error, which the bounds' margin covers.
 __device__ __forceinline__ float grid_inv(float d) {
-    return __frcp_rn(fabsf(d) > 1e-36f ? d : copysignf(1e-36f, d));
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) > 1e-36f ? d : copysignf(1e-36f, d)));
+    return r;
 }
 
 // A lane without a ray.
@@ -567,6 +569,12 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     stack[1] = make_uint2(__float_as_uint(from), 0u);
     s.node = meets ? root : REF_NONE;
     s.leaf = REF_NONE;
+}
+
+// tau of a hit at t, widened by the prune slack.
+__device__ __forceinline__ float compact_cap(float t, float from, float scale) {
+    const float tau = __fsub_ru(t, from);
+    return __fmul_ru(__fmaf_ru(__fadd_ru(fabsf(t), tau), PRUNE_SLACK - 1.0f, tau), scale);
 }
 
 // A leaf that is next becomes the lane's parked leaf if it has none (a node of
@@ -726,9 +734,7 @@ __device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, u
                     s.best_u = u;
                     s.best_v = v;
                     s.best_prim = prim;
-                    const float tau = __fsub_ru(t, __uint_as_float(e1.x));
-                    s.tcap = __fmul_ru(__fmaf_ru(__fadd_ru(fabsf(t), tau), PRUNE_SLACK - 1.0f, tau),
-                                       __uint_as_float(e0.y));
+                    s.tcap = compact_cap(t, __uint_as_float(e1.x), __uint_as_float(e0.y));
                     if (ANY) ray_none(s, stack_base);
                 }
             }
@@ -843,6 +849,159 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace(TraceArgs a) {
     }
     store_hit(a, i, s);
     add_counts<COUNT>(a, cn);
+}
+
+// ------------------------------------------------- four lanes per ray
+//
+// For wavefronts too small to fill the GPU a trace lasts as long as its longest
+// ray, and that ray as long as its chain of dependent steps.  Here four lanes
+// share a ray: each tests one child of a compact node and keeps the pending
+// children that it met on a stack of its own, and each tests one
+// triangle of a leaf, so that a step is a third of the instructions of
+// node_step and a leaf a single test.  All four hold the ray; minima over the quad
+// (two shuffles) pick the next subtree: the nearest child met, else the topmost
+// entry of the deepest level, ordered by one 32-bit key:
+//   63 - level, then 22 bits of the entry distance (rounded down), then the lane
+// The deepest level first makes it a depth-first walk, so a lane's stack holds at
+// most one entry per level.  Bound by the latency of that chain (a load from L2, two
+// shuffles and about 80 instructions a step); as throughput it is worse (0.96M
+// rays: 563 against 321 us), so launch_layout keeps it to small wavefronts.
+// (Prefetching the met children's nodes: no change at 4,096 rays, 4 % slower at 65,536.)
+constexpr int QUAD_SLACK = 8;  // lanes that may still descend when the triangles are tested (0: 5 % slower, 16: 1 %)
+constexpr uint64_t QUAD_MAX_N = 80000;
+constexpr uint32_t QUAD_MAX_LEVEL = 60;
+constexpr uint32_t QUAD_NONE = 0xFFFFFFFFu;
+
+__device__ __forceinline__ uint32_t quad_min(uint32_t v) {
+    v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, 1));
+    return min(v, __shfl_xor_sync(0xFFFFFFFFu, v, 2));
+}
+
+// Lower bound of the entry distance in a key.
+__device__ __forceinline__ float quad_distance(uint32_t key) { return __uint_as_float((key & 0x00FFFFFCu) << 6); }
+
+template <bool ANY>
+__global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const uint32_t lane = threadIdx.x & 31, child = lane & 3;
+    uint64_t i = (uint64_t)blockIdx.x * (TRACE_BLOCK / 4) + threadIdx.x / 4;
+    CompactState s;
+    uint2 aux[COMPACT_SLOTS], stack[STACK];
+    s.node = s.leaf = REF_NONE;
+    s.best_prim = -1;
+    const uint4 *nodes;
+    const float4 *tris;
+    bool have = i < a.n;
+    if (have) {
+        if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end, as the other traces
+        have = start_ray<false, COMPACT>(a, i, s, aux, nodes, tris);
+    }
+    const float tmin = __uint_as_float(aux[0].x), scale = __uint_as_float(aux[0].y), from = __uint_as_float(aux[1].x);
+    uint32_t level = 1;  // of the current node's children
+    uint32_t top_ref = REF_NONE, top_key = QUAD_NONE;
+    int sp = 0;
+    bool owner = false;  // this lane found the quad's best hit
+    // drops the topmost entry, and those below it beyond the best hit
+    auto pop = [&]() {
+        do {
+            --sp;
+            const uint2 e = sp > 0 ? stack[sp - 1] : make_uint2(REF_NONE, QUAD_NONE);
+            top_ref = e.x;
+            top_key = e.y;
+        } while (sp > 0 && quad_distance(top_key) > s.tcap);
+    };
+    bool live = have && (s.node != REF_NONE || s.leaf != REF_NONE);
+    while (__any_sync(FULL, live)) {
+        bool more;
+        do {
+            if (s.leaf == REF_NONE && s.node != REF_NONE && (s.node & REF_LEAF)) {  // park
+                s.leaf = s.node;
+                s.node = REF_NONE;
+            }
+            const bool internal = !(s.node & REF_LEAF);
+            uint32_t key = QUAD_NONE, ref = REF_NONE;
+            if (internal) {
+                const uint32_t *w = reinterpret_cast<const uint32_t *>(a.cnodes) + 16 * (size_t)s.node;
+                const uint32_t wx = __ldg(w + 3 * child), wy = __ldg(w + 3 * child + 1), wz = __ldg(w + 3 * child + 2);
+                ref = __ldg(w + 12 + child);
+                float tn, tf;
+                compact_child(s, wx, wy, wz, tn, tf);
+                if (tn < tf) key = ((63u - level) << 24) | ((__float_as_uint(tn) >> 6) & 0x00FFFFFCu) | child;
+            }
+            const bool met = key != QUAD_NONE;
+            const bool wants = internal || s.node == REF_NONE;  // not held up by a second leaf
+            if (!met) {
+                key = wants ? top_key : QUAD_NONE;
+                ref = top_ref;
+            }
+            const uint32_t best = quad_min(key);
+            const uint32_t next = __shfl_sync(FULL, ref, (lane & ~3u) | (best & 3u));
+            if (met && key != best) {  // another child is nearer: pending
+                stack[sp++] = make_uint2(ref, key);
+                top_ref = ref;
+                top_key = key;
+            } else if (!met && key == best && key != QUAD_NONE) {
+                pop();
+            }
+            if (wants) {
+                s.node = best != QUAD_NONE ? next : REF_NONE;
+                level = 64u - (best >> 24);
+            }
+            if (s.leaf == REF_NONE && s.node != REF_NONE && (s.node & REF_LEAF)) {
+                s.leaf = s.node;
+                s.node = REF_NONE;
+            }
+            more = s.leaf == REF_NONE && (s.node != REF_NONE);
+        } while (__popc(__ballot_sync(FULL, more)) > (ANY ? 0 : QUAD_SLACK));
+        // every lane one triangle of its quad's parked leaf
+        const bool at_leaf = s.leaf != REF_NONE;
+        float t = 0.0f, u = 0.0f, v = 0.0f;
+        int32_t prim = 0x7FFFFFFF;
+        bool hit = false;
+        if (at_leaf && child <= ((s.leaf >> 29) & 3u)) {
+            const float4 *rec = tris + 3 * (size_t)((s.leaf & REF_TRI_MASK) + child);
+            const float4 A = __ldg(rec), E1 = __ldg(rec + 1), E2 = __ldg(rec + 2);
+            const int32_t id = __float_as_int(A.w);
+            if (intersect(s.ox, s.oy, s.oz, s.dx, s.dy, s.dz, A, E1, E2, t, u, v) && t > tmin &&
+                (t < s.best_t || (t == s.best_t && id < s.best_prim))) {
+                hit = true;
+                prim = id;
+            }
+        }
+        if (at_leaf) s.leaf = REF_NONE;
+        if (__any_sync(FULL, hit)) {
+            // the quad's smallest (t, triangle id)
+            float bt = hit ? t : __int_as_float(0x7F800000);
+            bt = fminf(bt, __shfl_xor_sync(FULL, bt, 1));
+            bt = fminf(bt, __shfl_xor_sync(FULL, bt, 2));
+            const bool tied = hit && t == bt;
+            int32_t bp = tied ? prim : 0x7FFFFFFF;
+            bp = min(bp, __shfl_xor_sync(FULL, bp, 1));
+            bp = min(bp, __shfl_xor_sync(FULL, bp, 2));
+            if (bp != 0x7FFFFFFF) {
+                s.best_t = bt;
+                s.best_prim = bp;
+                owner = tied && prim == bp;
+                if (owner) {
+                    s.best_u = u;
+                    s.best_v = v;
+                }
+                s.tcap = compact_cap(bt, from, scale);
+                if (ANY) {
+                    s.node = REF_NONE;
+                    sp = 0;
+                    top_key = QUAD_NONE;
+                } else if (sp > 0 && quad_distance(top_key) > s.tcap) {
+                    pop();
+                }
+            }
+        }
+        // a quad lives while it has a node, a leaf or a pending entry
+        const uint32_t pending = __ballot_sync(FULL, sp > 0);
+        live = s.node != REF_NONE || s.leaf != REF_NONE || ((pending >> (lane & ~3u)) & 15u);
+    }
+    if (!have) return;
+    if (s.best_prim >= 0 ? owner : child == 0) store_hit(a, i, s);
 }
 
 // Persistent variant with ray replacement (Aila & Laine 2009, "replacing
@@ -992,6 +1151,16 @@ cudaError_t launch_layout(cudaStream_t s, const TraceArgs &a, bool pool) {
     if constexpr (!CNT) {
         const int depth = pool && !ANY ? a.stack : STACK;
         if (a.cstack <= (uint32_t)depth) {
+            if constexpr (!MULTI) {
+                // Four lanes per ray where the rays do not fill the GPU (whole call, one
+                // lane against four: 4,096 rays 84 / 73 us, 20,000 84 / 67, 65,536 97 / 83,
+                // 40,000 unsorted 56 / 45, 30,000 shadow rays 79 / 71; 100,000 113 / 115,
+                // unsorted 68 / 77); a walk's levels are at most its stack entries.
+                if (a.quads && a.n <= QUAD_MAX_N && a.cstack <= QUAD_MAX_LEVEL) {
+                    k_trace_quad<ANY><<<(unsigned)((a.n + TRACE_BLOCK / 4 - 1) / (TRACE_BLOCK / 4)), TRACE_BLOCK, 0, s>>>(a);
+                    return cudaGetLastError();
+                }
+            }
             if (pool) return launch_pool_shaped<ANY, CNT, COMPACT, MULTI>(s, a);
             k_trace<ANY, CNT, COMPACT, MULTI><<<(unsigned)((a.n + TRACE_BLOCK - 1) / TRACE_BLOCK), TRACE_BLOCK, 0, s>>>(a);
             return cudaGetLastError();

@@ -33,7 +33,7 @@ def _check(ctx, tris, org, dir_, layout="exact"):
         hcc.hcc_bvh_destroy(h)
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1000, 38912, 155649, 160000])
+@pytest.mark.parametrize("n", [1, 2, 7, 31, 32, 33, 1000, 38912, 80000, 80001, 155649, 160000])
 def test_partial_warps_and_first_refills(ctx, n):
     """Wavefronts that end inside a warp, and around the first slots taken by refilling."""
     tris = gen.random_tris(3, 60, mu=-1.5)
