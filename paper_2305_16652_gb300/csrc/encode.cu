@@ -196,44 +196,6 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_hcc(const 
     }
 }
 
-// TwoPoint: o and t = o + L d (one fused multiply-add per axis) normalised
-// to the scene box, quantised to b bits, Morton-interleaved most significant
-// level first in the order o.x o.y o.z t.x t.y t.z, left-justified in k bits.
-template <typename K>
-__global__ void __launch_bounds__(ENC_BLOCK) k_encode_twopoint(const float4 *__restrict__ org,
-                                                               const float4 *__restrict__ dir, uint64_t n, uint32_t rs,
-                                                               float lox, float loy, float loz, float ex, float ey,
-                                                               float ez, float L, uint32_t key_bits,
-                                                               K *__restrict__ keys) {
-    const uint32_t b = key_bits / 6;
-    const float levels = (float)(1u << b);  // exact power of two (b <= 10)
-    const uint32_t qmax = b ? ((1u << b) - 1u) : 0u;
-    const uint32_t pad = key_bits - 6 * b;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float4 o = __ldcs(org + i * rs);
-        const float4 d = __ldcs(dir + i * rs);
-        const float p[6] = {o.x, o.y, o.z, __fmaf_rn(L, d.x, o.x), __fmaf_rn(L, d.y, o.y), __fmaf_rn(L, d.z, o.z)};
-        const float lo[3] = {lox, loy, loz}, ext[3] = {ex, ey, ez};
-        uint32_t q[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const int a = c % 3;
-            float u = (ext[a] == 0.0f) ? 0.0f : __fdiv_rn(__fsub_rn(p[c], lo[a]), ext[a]);
-            u = fminf(fmaxf(u, 0.0f), 1.0f);
-            const uint32_t qi = __float2uint_rz(__fmul_rn(u, levels));
-            q[c] = qi < qmax ? qi : qmax;
-        }
-        K key = 0;
-        for (int j = (int)b - 1; j >= 0; --j) {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) key = (key << 1) | (K)((q[c] >> j) & 1u);
-        }
-        if (pad) key <<= pad;
-        __stcs(keys + i, key);
-    }
-}
-
 // Normalise p to the box [lo, lo + ext], clamp to [0, 1], quantise to b bits.
 __device__ __forceinline__ uint32_t quantise(float p, float lo, float ext, uint32_t b) {
     if (b == 0) return 0u;
@@ -244,15 +206,65 @@ __device__ __forceinline__ uint32_t quantise(float p, float lo, float ext, uint3
     return q < qmax ? q : qmax;
 }
 
-// Morton interleave, most significant level first, coordinates in order.
+// The bits of x (below 2^5 for M = 6, 2^10 for M = 3 and 2) M apart.  M = 6: copies
+// of the five bits five apart do not overlap, so one multiplication puts bit j
+// of copy j at 6 j; otherwise the bits are moved apart in halving groups.
+template <int M>
+__device__ __forceinline__ uint32_t spread(uint32_t x) {
+    if (M == 6) return (x * 0x00108421u) & 0x01041041u;
+    if (M == 3) {
+        x = (x | (x << 16)) & 0x030000FFu;
+        x = (x | (x << 8)) & 0x0300F00Fu;
+        x = (x | (x << 4)) & 0x030C30C3u;
+        return (x | (x << 2)) & 0x09249249u;
+    }
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+
+// Morton interleave, most significant level first, coordinates in order: the
+// bits of all coordinates 30 key bits at a time.  (One key bit at a time took 51
+// us for 4M 48-bit TwoPoint keys.)
 template <typename K, int M>
 __device__ __forceinline__ K interleave(const uint32_t (&q)[M], uint32_t b) {
+    constexpr uint32_t GROUP = M == 6 ? 5 : 10;  // bits of a coordinate per group
     K key = 0;
-    for (int j = (int)b - 1; j >= 0; --j) {
 #pragma unroll
-        for (int c = 0; c < M; ++c) key = (key << 1) | (K)((q[c] >> j) & 1u);
+    for (uint32_t g = 0; g < (sizeof(K) == 8 ? 3u : 1u); ++g) {
+        if (g * GROUP >= b) break;
+        uint32_t part = 0;
+#pragma unroll
+        for (int c = 0; c < M; ++c) part |= spread<M>((q[c] >> (g * GROUP)) & ((1u << GROUP) - 1u)) << (M - 1 - c);
+        key |= (K)part << (g * GROUP * M);
     }
     return key;
+}
+
+// TwoPoint: o and t = o + L d (one fused multiply-add per axis) normalised
+// to the scene box, quantised to b bits, Morton-interleaved most significant
+// level first in the order o.x o.y o.z t.x t.y t.z, left-justified in k bits.
+template <typename K>
+__global__ void __launch_bounds__(ENC_BLOCK) k_encode_twopoint(const float4 *__restrict__ org,
+                                                               const float4 *__restrict__ dir, uint64_t n, uint32_t rs,
+                                                               float lox, float loy, float loz, float ex, float ey,
+                                                               float ez, float L, uint32_t key_bits,
+                                                               K *__restrict__ keys) {
+    const uint32_t b = key_bits / 6, pad = key_bits - 6 * b;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const float4 o = __ldcs(org + i * rs);
+        const float4 d = __ldcs(dir + i * rs);
+        const float p[6] = {o.x, o.y, o.z, __fmaf_rn(L, d.x, o.x), __fmaf_rn(L, d.y, o.y), __fmaf_rn(L, d.z, o.z)};
+        const float lo[3] = {lox, loy, loz}, ext[3] = {ex, ey, ez};
+        uint32_t q[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) q[c] = quantise(p[c], lo[c % 3], ext[c % 3], b);
+        K key = interleave<K, 6>(q, b);
+        if (pad) key <<= pad;
+        __stcs(keys + i, key);
+    }
 }
 
 // Octahedral map of a direction: L1-normalise, fold the lower hemisphere

@@ -146,27 +146,38 @@ __device__ __forceinline__ K key_mask(uint32_t key_bits) {
 }
 
 // Exclusive scan of each pass's histogram, pass activity and the buffer plan
-// (run by one block of RADIX threads: the last k_hist block).
-__device__ void plan_passes(SortHeader *h, int passes, uint64_t n) {
-    __shared__ uint32_t s_scan[RADIX];
-    __shared__ int s_trivial[MAX_PASSES];
-    const int t = threadIdx.x;
-    for (int p = 0; p < passes; ++p) {
-        const uint32_t c = ld_relaxed(&h->hist[p][t]);
-        s_scan[t] = c;
-        __syncthreads();
-        for (int off = 1; off < RADIX; off <<= 1) {
-            const uint32_t v = t >= off ? s_scan[t - off] : 0u;
-            __syncthreads();
-            s_scan[t] += v;
-            __syncthreads();
+// (run by one block of RADIX threads, the last k_hist block, while nothing else
+// runs: all P scans go together, one barrier for all warps' sums).
+template <int P>
+__device__ void plan_passes(SortHeader *h, uint64_t n) {
+    __shared__ uint32_t s_sum[P][RADIX / 32];
+    __shared__ int s_trivial[P];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint32_t c[P], incl[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) incl[p] = c[p] = ld_relaxed(&h->hist[p][t]);
+    if (t < P) s_trivial[t] = 0;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl[p], off);
+            if (lane >= off) incl[p] += v;
         }
-        h->start[p][t] = s_scan[t] - c;
-        if (t == 0) s_trivial[p] = 0;
-        __syncthreads();
-        if ((uint64_t)c == n) s_trivial[p] = 1;
-        __syncthreads();
     }
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+        if (lane == 31) s_sum[p][warp] = incl[p];
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        uint32_t before = 0;
+        for (int w = 0; w < warp; ++w) before += s_sum[p][w];
+        h->start[p][t] = before + incl[p] - c[p];
+        if ((uint64_t)c[p] == n) s_trivial[p] = 1;
+    }
+    __syncthreads();
+    constexpr int passes = P;
     if (t == 0) {
         int act[MAX_PASSES], m = 0;
         for (int p = 0; p < passes; ++p) {
@@ -285,7 +296,7 @@ __global__ void __launch_bounds__(HIST_BLOCK) k_hist(const K *__restrict__ keys,
     __syncthreads();
     if (s_last) {
         __threadfence();
-        plan_passes(h, P, n);
+        plan_passes<P>(h, n);
     }
 }
 

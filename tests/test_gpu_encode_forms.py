@@ -73,3 +73,21 @@ def test_mlhcc_keys(env, top, low, k):
     got = keys.cpu().numpy().view(np.uint32 if k <= 32 else np.uint64).astype(np.uint64)
     ref = oracle.encode_mlhcc(org, dir_, tf, bvh.lo[top_ids], bvh.hi[top_ids], bvh.lo[low_ids], bvh.hi[low_ids], k)
     assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 6, 12, 29, 30, 31, 32, 33, 36, 47, 48, 59, 60, 61, 63, 64])
+def test_morton_keys(env, k):
+    """Every number of bits per coordinate around the groups that are interleaved at once."""
+    ctx, bvh, h = env
+    n = 4_001
+    org, dir_ = _rays(n, k, False)
+    o, d = torch.from_numpy(org).to(DEV), torch.from_numpy(dir_).to(DEV)
+    lo, hi = bvh.lo[0], bvh.hi[0]
+    for method, ref in (("twopoint", oracle.encode_twopoint(org, dir_, lo, hi, k)),
+                        ("origin", oracle.encode_origin(org, lo, hi, k)),
+                        ("origin_dir", oracle.encode_origin_dir(org, dir_, lo, hi, k))):
+        keys = torch.zeros(n, dtype=torch.int32 if k <= 32 else torch.int64, device=DEV)
+        hcc.hcc_encode(ctx, method, h, None, o, d, k, keys)
+        hcc.hcc_sync(ctx)
+        got = keys.cpu().numpy().view(np.uint32 if k <= 32 else np.uint64).astype(np.uint64)
+        assert np.array_equal(got, ref), method
