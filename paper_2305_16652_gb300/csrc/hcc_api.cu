@@ -28,15 +28,15 @@ struct DevBuf {
 };
 
 // Rays per chunk and lanes (contexts with their own streams) of the
-// pipelined hcc_run_host.
-constexpr uint64_t HOST_CHUNK = 1ull << 22;
+// pipelined hcc_run_host, and the most rays that go through in one pass.
+constexpr uint64_t HOST_CHUNK = 1ull << 21;
+constexpr uint64_t HOST_ONE_PASS = 3ull << 19;
 constexpr uint32_t HOST_LANES = 2;
-// The first chunks are a quarter and a half as large, so the first kernels
-// start sooner while the next copies catch up (1M, 2M, then 4M rays: 5.81 ms
-// for the room's 16.6M rays against 5.88 with 2M then 4M, 5.98 with 1M then 4M).
-static uint64_t host_chunk_rays(uint64_t c, uint64_t rem) {
-    return std::min(c == 0 ? HOST_CHUNK / 4 : c == 1 ? HOST_CHUNK / 2 : HOST_CHUNK, rem);
-}
+// The first chunk is half as large, so the first kernels start sooner.  (6M rays:
+// 1.99 ms with chunks of 1M, then 2M; 2.24 with 1M, 2M, then 4M; 2.16 with 1M
+// throughout; 16.6M rays 4.88, 4.87 and 5.31.  Two passes beat one from 1.5M
+// rays up: 1.8M 0.88 against 0.98 ms, 3.5M 1.35 against 1.75.)
+static uint64_t host_chunk_rays(uint64_t c, uint64_t rem) { return std::min(c == 0 ? HOST_CHUNK / 2 : HOST_CHUNK, rem); }
 
 struct hcc_ctx {
     int device = 0;
@@ -1645,7 +1645,7 @@ hcc_status hcc_run_host(hcc_ctx *ctx, hcc_method method, const hcc_bvh *bvh, con
     DeviceGuard g(ctx->device);
     hcc_status st;
     cudaError_t e;
-    if (n <= HOST_CHUNK) {
+    if (n <= HOST_ONE_PASS) {
         // one pass on the context's stream
         if ((st = ensure(ctx, ctx->in_org, n * 16, "input rays")) != HCC_OK) return st;
         if ((st = ensure(ctx, ctx->in_dir, n * 16, "input rays")) != HCC_OK) return st;
