@@ -689,6 +689,18 @@ __device__ __forceinline__ void node_step(CompactState &s, const uint4 *__restri
     push_node<true>(s, r1, n1);
 }
 
+// A read-only 16-byte load that L1 evicts first: triangles are met by few rays
+// each and would push out nodes and stacks (16.6M rays in HCC order, whole
+// bounce: 3.92 -> 3.87 ms, 2.1M unsorted 434 -> 426 us; not cached in L1 at all: 4.65 ms and
+// 604 us; nodes evicted last on top: no change).
+__device__ __forceinline__ float4 ldg_first(const float4 *p) {
+    float4 r;
+    asm("ld.global.nc.L1::evict_first.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+        : "l"(p));
+    return r;
+}
+
 // One round over compact nodes, run by the whole warp together (a lane without
 // a ray takes part in the votes only): node steps until all but COMPACT_SLACK of
 // the lanes that could go on hold a parked leaf, then triangle tests, one triangle
@@ -716,7 +728,7 @@ __device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, u
     while (__any_sync(FULL, s.leaf != REF_NONE)) {
         if (s.leaf != REF_NONE) {
             const float4 *rec = tris + 3 * (size_t)(s.leaf & REF_TRI_MASK);
-            const float4 A = __ldg(rec), E1 = __ldg(rec + 1), E2 = __ldg(rec + 2);
+            const float4 A = ldg_first(rec), E1 = ldg_first(rec + 1), E2 = ldg_first(rec + 2);
             // the next triangle of the leaf, or the next leaf
             if (s.leaf & ~(REF_LEAF | REF_TRI_MASK)) {
                 s.leaf -= REF_TRI_MASK;
