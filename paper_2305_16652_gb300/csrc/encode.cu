@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_hcc(const 
                                                           const float4 *__restrict__ cut, uint32_t used,
                                                           uint32_t key_bits, K *__restrict__ keys) {
     __shared__ float4 s_pairs[MAX_CUT_BITS / 2 * 6];
-    const bool ordered = __syncthreads_and(stage_boxes(s_pairs, cut, used));
+    const bool ordered = __syncthreads_and(stage_boxes(s_pairs, cut, used));  // a cut is not written after its creation
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const SlabRay r = slab_ray(__ldcs(org + i * rs), __ldcs(dir + i * rs), ordered);
@@ -252,6 +253,7 @@ __global__ void __launch_bounds__(ENC_BLOCK) k_encode_twopoint(const float4 *__r
                                                                float ez, float L, uint32_t key_bits,
                                                                K *__restrict__ keys) {
     const uint32_t b = key_bits / 6, pad = key_bits - 6 * b;
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float4 o = __ldcs(org + i * rs);
@@ -292,6 +294,7 @@ __global__ void __launch_bounds__(ENC_BLOCK) k_encode_origin(const float4 *__res
                                                              float loy, float loz, float ex, float ey, float ez,
                                                              uint32_t key_bits, K *__restrict__ keys) {
     const uint32_t b = key_bits / 3, pad = key_bits - 3 * b;
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float4 o = __ldcs(org + i * rs);
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(ENC_BLOCK) k_encode_origin_dir(const float4 *_
                                                                  K *__restrict__ keys) {
     const uint32_t bd = key_bits / 6, bo = (key_bits - 2 * bd) / 3;
     const uint32_t pad = key_bits - (3 * bo + 2 * bd);
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float4 o = __ldcs(org + i * rs);
@@ -390,6 +394,7 @@ __global__ void __launch_bounds__(ENC_BLOCK) k_encode_multi(const float4 *__rest
                                                             const SceneDesc *__restrict__ scenes,
                                                             const uint64_t *__restrict__ offsets, uint32_t num_scenes,
                                                             uint32_t key_bits, K *__restrict__ keys) {
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint32_t s = scene_of(offsets, num_scenes, i);
@@ -420,6 +425,7 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_multi_hcc(
                                                                 uint32_t num_scenes, uint32_t key_bits,
                                                                 K *__restrict__ keys) {
     __shared__ float4 s_pairs[MAX_CUT_BITS / 2 * 6];
+    wait_for_previous();
     const uint64_t run = (n + gridDim.x - 1) / gridDim.x;
     uint64_t i0 = run * blockIdx.x;
     const uint64_t end = i0 + run < n ? i0 + run : n;
@@ -447,19 +453,18 @@ cudaError_t launch_encode_multi(cudaStream_t s, int method, const float4 *org, c
                                 uint32_t key_bits, uint32_t total_bits, void *keys) {
     if (n == 0) return cudaSuccess;
     const int grid = encode_grid(n, ENC_BLOCK, 8);
-#define HCC_ENC_MULTI(K, M) \
-    k_encode_multi<K, M><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, scenes, offsets, num_scenes, key_bits, (K *)keys)
-#define HCC_ENC_MULTI_K(K)                                                      \
-    do {                                                                        \
-        if (method == HCC_METHOD_HCC)                                           \
-            k_encode_multi_hcc<K><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, scenes, offsets, num_scenes, key_bits, \
-                                                             (K *)keys);        \
-        else if (method == HCC_METHOD_TWOPOINT)                                 \
-            HCC_ENC_MULTI(K, HCC_METHOD_TWOPOINT);                              \
-        else if (method == HCC_METHOD_ORIGIN)                                   \
-            HCC_ENC_MULTI(K, HCC_METHOD_ORIGIN);                                \
-        else                                                                    \
-            HCC_ENC_MULTI(K, HCC_METHOD_ORIGIN_DIR);                            \
+#define HCC_ENC_MULTI(K, KERNEL)                                                                                    \
+    return launch_early(KERNEL, grid, ENC_BLOCK, 0, s, org, dir, n, rs, scenes, offsets, num_scenes, key_bits, (K *)keys)
+#define HCC_ENC_MULTI_K(K)                                            \
+    do {                                                              \
+        if (method == HCC_METHOD_HCC)                                 \
+            HCC_ENC_MULTI(K, k_encode_multi_hcc<K>);                  \
+        else if (method == HCC_METHOD_TWOPOINT)                       \
+            HCC_ENC_MULTI(K, (k_encode_multi<K, HCC_METHOD_TWOPOINT>)); \
+        else if (method == HCC_METHOD_ORIGIN)                         \
+            HCC_ENC_MULTI(K, (k_encode_multi<K, HCC_METHOD_ORIGIN>)); \
+        else                                                          \
+            HCC_ENC_MULTI(K, (k_encode_multi<K, HCC_METHOD_ORIGIN_DIR>)); \
     } while (0)
     if (total_bits <= 32)
         HCC_ENC_MULTI_K(uint32_t);
@@ -467,7 +472,6 @@ cudaError_t launch_encode_multi(cudaStream_t s, int method, const float4 *org, c
         HCC_ENC_MULTI_K(uint64_t);
 #undef HCC_ENC_MULTI_K
 #undef HCC_ENC_MULTI
-    return cudaGetLastError();
 }
 
 cudaError_t launch_key_stats(cudaStream_t s, const void *keys, uint32_t key_bits, const uint32_t *perm, uint64_t n,
@@ -489,12 +493,10 @@ cudaError_t launch_encode_origin(cudaStream_t s, const float4 *org, uint64_t n, 
     if (n == 0) return cudaSuccess;
     const int grid = encode_grid(n, ENC_BLOCK, 8);
     if (key_bits <= 32)
-        k_encode_origin<uint32_t><<<grid, ENC_BLOCK, 0, s>>>(org, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1], ext[2],
-                                                             key_bits, (uint32_t *)keys);
-    else
-        k_encode_origin<uint64_t><<<grid, ENC_BLOCK, 0, s>>>(org, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1], ext[2],
-                                                             key_bits, (uint64_t *)keys);
-    return cudaGetLastError();
+        return launch_early(k_encode_origin<uint32_t>, grid, ENC_BLOCK, 0, s, org, n, rs, lo[0], lo[1], lo[2], ext[0],
+                            ext[1], ext[2], key_bits, (uint32_t *)keys);
+    return launch_early(k_encode_origin<uint64_t>, grid, ENC_BLOCK, 0, s, org, n, rs, lo[0], lo[1], lo[2], ext[0],
+                        ext[1], ext[2], key_bits, (uint64_t *)keys);
 }
 
 cudaError_t launch_encode_origin_dir(cudaStream_t s, const float4 *org, const float4 *dir, uint64_t n, uint32_t rs,
@@ -502,12 +504,10 @@ cudaError_t launch_encode_origin_dir(cudaStream_t s, const float4 *org, const fl
     if (n == 0) return cudaSuccess;
     const int grid = encode_grid(n, ENC_BLOCK, 8);
     if (key_bits <= 32)
-        k_encode_origin_dir<uint32_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1],
-                                                                 ext[2], key_bits, (uint32_t *)keys);
-    else
-        k_encode_origin_dir<uint64_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1],
-                                                                 ext[2], key_bits, (uint64_t *)keys);
-    return cudaGetLastError();
+        return launch_early(k_encode_origin_dir<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
+                            ext[0], ext[1], ext[2], key_bits, (uint32_t *)keys);
+    return launch_early(k_encode_origin_dir<uint64_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
+                        ext[0], ext[1], ext[2], key_bits, (uint64_t *)keys);
 }
 
 namespace {
@@ -537,6 +537,7 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_mlhcc(cons
         }
     }
     ordered = __syncthreads_and(ordered);
+    wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const SlabRay r = slab_ray(__ldcs(org + i * rs), __ldcs(dir + i * rs), ordered);
@@ -629,15 +630,13 @@ cudaError_t launch_encode_mlhcc(cudaStream_t s, const float4 *org, const float4 
     if (key_bits <= 32) {
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_encode_mlhcc<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_encode_mlhcc<uint32_t><<<grid, ENC_BLOCK, smem, s>>>(org, dir, n, rs, top, ntop, top_field, low, low_field,
-                                                              key_bits, (uint32_t *)keys);
-    } else {
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(k_encode_mlhcc<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_encode_mlhcc<uint64_t><<<grid, ENC_BLOCK, smem, s>>>(org, dir, n, rs, top, ntop, top_field, low, low_field,
-                                                              key_bits, (uint64_t *)keys);
+        return launch_early(k_encode_mlhcc<uint32_t>, grid, ENC_BLOCK, smem, s, org, dir, n, rs, top, ntop, top_field, low,
+                            low_field, key_bits, (uint32_t *)keys);
     }
-    return cudaGetLastError();
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_encode_mlhcc<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return launch_early(k_encode_mlhcc<uint64_t>, grid, ENC_BLOCK, smem, s, org, dir, n, rs, top, ntop, top_field, low,
+                        low_field, key_bits, (uint64_t *)keys);
 }
 
 cudaError_t launch_encode_ppc(cudaStream_t s, const float4 *org, const float4 *dir, uint64_t n, uint32_t rs, const uint4 *nodes,
@@ -664,10 +663,10 @@ cudaError_t launch_encode_hcc(cudaStream_t s, const float4 *org, const float4 *d
     if (used > MAX_CUT_BITS) used = MAX_CUT_BITS;
     const int grid = encode_grid(n, ENC_BLOCK, ENC_BOX_BLOCKS);
     if (key_bits <= 32)
-        k_encode_hcc<uint32_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, cut_boxes, used, key_bits, (uint32_t *)keys);
-    else
-        k_encode_hcc<uint64_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, cut_boxes, used, key_bits, (uint64_t *)keys);
-    return cudaGetLastError();
+        return launch_early(k_encode_hcc<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, cut_boxes, used, key_bits,
+                            (uint32_t *)keys);
+    return launch_early(k_encode_hcc<uint64_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, cut_boxes, used, key_bits,
+                        (uint64_t *)keys);
 }
 
 cudaError_t launch_encode_twopoint(cudaStream_t s, const float4 *org, const float4 *dir, uint64_t n, uint32_t rs,
@@ -675,12 +674,10 @@ cudaError_t launch_encode_twopoint(cudaStream_t s, const float4 *org, const floa
     if (n == 0) return cudaSuccess;
     const int grid = encode_grid(n, ENC_BLOCK, 8);
     if (key_bits <= 32)
-        k_encode_twopoint<uint32_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1],
-                                                               ext[2], L, key_bits, (uint32_t *)keys);
-    else
-        k_encode_twopoint<uint64_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, lo[0], lo[1], lo[2], ext[0], ext[1],
-                                                               ext[2], L, key_bits, (uint64_t *)keys);
-    return cudaGetLastError();
+        return launch_early(k_encode_twopoint<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
+                            ext[0], ext[1], ext[2], L, key_bits, (uint32_t *)keys);
+    return launch_early(k_encode_twopoint<uint64_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
+                        ext[0], ext[1], ext[2], L, key_bits, (uint64_t *)keys);
 }
 
 }  // namespace hcc

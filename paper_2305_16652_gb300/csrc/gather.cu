@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(GATHER_BLOCK) k_gather(const float4 *__restric
                                                          float4 *__restrict__ out_org, float4 *__restrict__ out_dir,
                                                          uint32_t out_rs, uint64_t n, uint32_t *err) {
     const uint64_t base = (uint64_t)blockIdx.x * (GATHER_BLOCK * GATHER_RAYS) + threadIdx.x;
+    wait_for_previous();
     uint32_t src[GATHER_RAYS];
 #pragma unroll
     for (int k = 0; k < GATHER_RAYS; ++k) {
@@ -88,13 +89,10 @@ cudaError_t launch_gather(cudaStream_t s, const float4 *in_org, const float4 *in
     if (n == 0) return cudaSuccess;
     const uint64_t per_block = (uint64_t)GATHER_BLOCK * GATHER_RAYS;
     const uint64_t blocks = (n + per_block - 1) / per_block;
-    if (is_record(in_org, in_dir, in_rs) && is_record(out_org, out_dir, out_rs))
-        k_gather<true><<<(unsigned)blocks, GATHER_BLOCK, 0, s>>>(in_org, in_dir, in_rs, in_n, perm, out_org, out_dir,
-                                                                 out_rs, n, err);
-    else
-        k_gather<false><<<(unsigned)blocks, GATHER_BLOCK, 0, s>>>(in_org, in_dir, in_rs, in_n, perm, out_org,
-                                                                  out_dir, out_rs, n, err);
-    return cudaGetLastError();
+    const auto kernel =
+        is_record(in_org, in_dir, in_rs) && is_record(out_org, out_dir, out_rs) ? k_gather<true> : k_gather<false>;
+    return launch_early(kernel, (unsigned)blocks, GATHER_BLOCK, 0, s, in_org, in_dir, in_rs, in_n, perm, out_org, out_dir,
+                        out_rs, n, err);
 }
 
 }  // namespace hcc

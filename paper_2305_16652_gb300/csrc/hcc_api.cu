@@ -41,8 +41,8 @@ static uint64_t host_chunk_rays(uint64_t c, uint64_t rem) { return std::min(c ==
 struct hcc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
-    uint32_t *d_err = nullptr;                 // device error word (16-byte allocation) ...
-    unsigned long long *d_work = nullptr;      // ... whose second half is the trace's slot counter
+    uint32_t *d_err = nullptr;                 // device error word, followed by ...
+    hcc::TraceWork *d_work = nullptr;          // ... the trace's counters
     hcc_trace_schedule schedule = HCC_TRACE_AUTO;
     float twopoint_fraction = 0.25f;            // TwoPoint length estimate / largest extent
     hcc::SortOptions sort_opt;                  // bounded-wait settings of this context's sorts
@@ -350,8 +350,8 @@ void cut_view(const hcc_cut *c, const float4 **boxes, uint32_t *on_device, int *
 
 }  // namespace hcc
 
-// Slot counter for the persistent trace, or NULL for one thread per ray.
-static unsigned long long *trace_work(const hcc_ctx *ctx, int any_hit) {
+// Counters for the persistent trace, or NULL for one thread per ray.
+static TraceWork *trace_work(const hcc_ctx *ctx, int any_hit) {
     const bool refill = ctx->schedule == HCC_TRACE_REFILL || (ctx->schedule == HCC_TRACE_AUTO && !any_hit);
     return refill ? ctx->d_work : nullptr;
 }
@@ -413,13 +413,13 @@ hcc_status hcc_create(hcc_ctx **out, int device, void *stream) {
     c->device = device;
     c->stream = static_cast<cudaStream_t>(stream);
     DeviceGuard g(device);
-    if (cudaMalloc(&c->d_err, 16) != cudaSuccess) {
+    if (cudaMalloc(&c->d_err, CTX_WORDS_BYTES) != cudaSuccess) {
         cudaGetLastError();
         delete c;
         return HCC_ERR_OOM;
     }
-    c->d_work = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(c->d_err) + 8);
-    if (cudaMemset(c->d_err, 0, 16) != cudaSuccess) {
+    c->d_work = trace_counters(c->d_err);
+    if (cudaMemset(c->d_err, 0, CTX_WORDS_BYTES) != cudaSuccess) {
         cudaFree(c->d_err);
         delete c;
         return HCC_ERR_CUDA;

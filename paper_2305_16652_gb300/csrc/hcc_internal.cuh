@@ -105,6 +105,29 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
     return r;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_early may start
+// while the last blocks of the kernel before it on the stream still run, and calls
+// wait_for_previous before it touches anything that one writes or reads (it
+// returns once the previous grid is done and its writes are visible; at once in a
+// kernel launched the ordinary way).
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s,
+                         Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // ------------------------------------------------------------------ launchers
 // All return the launch error (cudaSuccess when queued).
 
@@ -165,6 +188,17 @@ cudaError_t launch_gather(cudaStream_t s, const float4 *in_org, const float4 *in
                           const uint32_t *perm, float4 *out_org, float4 *out_dir, uint32_t out_rs, uint64_t n,
                           uint32_t *err);
 
+// Counters of the persistent trace, zero between traces: the last block of a
+// trace leaves them so.
+struct TraceWork {
+    unsigned long long next;  // next ray slot to hand out
+    uint32_t done;            // blocks that have finished
+    uint32_t pad;
+};
+// A context's device words: the error word, then the trace's counters.
+constexpr size_t CTX_WORDS_BYTES = 16 + sizeof(TraceWork);
+inline TraceWork *trace_counters(uint32_t *err) { return reinterpret_cast<TraceWork *>(err + 4); }
+
 struct TraceArgs {
     const uint4 *nodes = nullptr;  // 2 (quantised), 4 (exact) or 8 (wide) per node
     int layout = 0;          // 0 = 32-byte quantised, 1 = 64-byte exact, 2 = 128-byte wide
@@ -188,7 +222,7 @@ struct TraceArgs {
     const SceneDesc *scenes = nullptr;     // batch mode (NULL = single BVH above)
     const uint64_t *offsets = nullptr;     // scene s owns rays [offsets[s], offsets[s+1])
     uint32_t num_scenes = 0;
-    unsigned long long *work = nullptr;    // slot counter of the persistent trace (NULL: one thread per slot)
+    TraceWork *work = nullptr;             // counters of the persistent trace (NULL: one thread per slot)
     bool quads = false;                    // small wavefronts may be traced with four lanes per ray
     int block = 128;                       // closest-hit persistent trace: threads per block ...
     int stack = HCC_TRACE_STACK;           // ... and stack entries per ray (a supported shape)

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(SPAWN_BLOCK) k_spawn(const float4 *__restrict_
                                                        float4 *__restrict__ out_dir, uint32_t out_rs, uint32_t *err) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t sm = mix64(seed);
+    wait_for_previous();
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float4 o = in_org[i * in_rs], d = in_dir[i * in_rs];
         const int4 h = hits[i];
@@ -124,9 +125,8 @@ cudaError_t launch_spawn(cudaStream_t s, const float4 *in_org, const float4 *in_
     uint64_t blocks = (n + SPAWN_BLOCK - 1) / SPAWN_BLOCK;
     const uint64_t cap = (uint64_t)(sms > 0 ? sms : 1) * 8;
     if (blocks > cap) blocks = cap;
-    k_spawn<<<(unsigned)blocks, SPAWN_BLOCK, 0, s>>>(in_org, in_dir, in_rs, hits, n, scenes, offsets, num_scenes, seed,
-                                                     tmin, out_org, out_dir, out_rs, err);
-    return cudaGetLastError();
+    return launch_early(k_spawn, (unsigned)blocks, SPAWN_BLOCK, 0, s, in_org, in_dir, in_rs, hits, n, scenes, offsets,
+                        num_scenes, seed, tmin, out_org, out_dir, out_rs, err);
 }
 
 }  // namespace hcc

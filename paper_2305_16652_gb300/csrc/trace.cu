@@ -899,6 +899,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     const uint32_t lane = threadIdx.x & 31, child = lane & 3;
     uint64_t i = (uint64_t)blockIdx.x * (TRACE_BLOCK / 4) + threadIdx.x / 4;
+    wait_for_previous();
     CompactState s;
     uint2 aux[COMPACT_SLOTS], stack[STACK];
     s.node = s.leaf = REF_NONE;
@@ -1040,6 +1041,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
 template <bool ANY, bool COUNT, int LAYOUT, bool MULTI, int BLOCK, int STACKN>
 __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
     k_trace_pool(TraceArgs a) {
+    wait_for_previous();
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     const uint32_t lane = threadIdx.x & 31;
     uint32_t lt;
@@ -1061,7 +1063,7 @@ __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
         if (need && (busy == 0 || (uint32_t)__popc(need) >= refill_min)) {
             const int leader = __ffs(need) - 1;
             unsigned long long base = 0;
-            if ((int)lane == leader) base = atomicAdd(a.work, (unsigned long long)__popc(need));
+            if ((int)lane == leader) base = atomicAdd(&a.work->next, (unsigned long long)__popc(need));
             base = __shfl_sync(FULL, base, leader);
             if (want) {
                 const uint64_t at = base + __popc(need & lt);
@@ -1094,6 +1096,15 @@ __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
         }
     }
     add_counts<COUNT>(a, cn);
+    // the last block to finish clears the counters for the next trace
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&a.work->done, 1u) == gridDim.x - 1) {
+            a.work->next = 0;
+            a.work->done = 0;
+        }
+    }
 }
 
 }  // namespace
@@ -1128,10 +1139,7 @@ cudaError_t launch_pool(cudaStream_t s, const TraceArgs &a) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned cap = (unsigned)std::max(1, sms) * (unsigned)resident_blocks((const void *)kernel, BLOCK);
     const unsigned blocks = (unsigned)std::min<uint64_t>((a.n + BLOCK - 1) / BLOCK, cap);
-    cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    kernel<<<blocks, BLOCK, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_early(kernel, blocks, BLOCK, 0, s, a);
 }
 
 // The closest-hit persistent trace in the shape the context asks for; the
@@ -1171,8 +1179,8 @@ cudaError_t launch_layout(cudaStream_t s, const TraceArgs &a, bool pool) {
                 // 40,000 unsorted 56 / 45, 30,000 shadow rays 79 / 71; 100,000 113 / 115,
                 // unsorted 68 / 77); a walk's levels are at most its stack entries.
                 if (a.quads && a.n <= QUAD_MAX_N && a.cstack <= QUAD_MAX_LEVEL) {
-                    k_trace_quad<ANY><<<(unsigned)((a.n + TRACE_BLOCK / 4 - 1) / (TRACE_BLOCK / 4)), TRACE_BLOCK, 0, s>>>(a);
-                    return cudaGetLastError();
+                    return launch_early(k_trace_quad<ANY>, (unsigned)((a.n + TRACE_BLOCK / 4 - 1) / (TRACE_BLOCK / 4)),
+                                        TRACE_BLOCK, 0, s, a);
                 }
             }
             if (pool) return launch_pool_shaped<ANY, CNT, COMPACT, MULTI>(s, a);
