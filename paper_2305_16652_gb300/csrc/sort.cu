@@ -181,32 +181,25 @@ __device__ void plan_passes(SortHeader *h, uint64_t n) {
         if ((uint64_t)c[p] == n) s_trivial[p] = 1;
     }
     __syncthreads();
-    constexpr int passes = P;
-    if (t == 0) {
-        int act[MAX_PASSES], m = 0;
-        for (int p = 0; p < passes; ++p) {
-            h->plan[p].active = 0;
-            if (!s_trivial[p]) act[m++] = p;
-        }
+    // thread p plans pass p from the set of active passes
+    const uint32_t active = __ballot_sync(0xFFFFFFFFu, lane < P && !s_trivial[lane < P ? lane : 0]);
+    if (t < P) {
+        const int m = __popc(active), idx = __popc(active & ((1u << t) - 1u));
         // wide passes alternate so that the last one reads the first buffer (its
         // ids are not in the permutation) and writes pairs to the second
-        const int wide = wide_passes(passes);
-        int lw = -1;  // last active wide pass
-        for (int idx = 0; idx < m; ++idx)
-            if (act[idx] < wide) lw = idx;
-        for (int idx = 0; idx < m; ++idx) {
-            PassPlan &pl = h->plan[act[idx]];
-            pl.active = 1;
-            pl.src = idx == 0 ? BUF_USER : h->plan[act[idx - 1]].dst;
-            pl.narrow = idx == lw && idx < m - 1;
-            if (idx == m - 1)
-                pl.dst = BUF_PERM;
-            else if (idx < lw)
-                pl.dst = (lw - 1 - idx) % 2 == 0 ? BUF_A : BUF_B;
-            else
-                pl.dst = (idx - lw) % 2 == 0 ? BUF_B : BUF_A;
-        }
-        h->identity = (m == 0);
+        const int lw = __popc(active & ((1u << wide_passes(P)) - 1u)) - 1;  // last active wide pass
+        auto target = [&](int i) {  // where active pass i writes
+            if (i == m - 1) return (int)BUF_PERM;
+            if (i < lw) return (lw - 1 - i) % 2 == 0 ? (int)BUF_A : (int)BUF_B;
+            return (i - lw) % 2 == 0 ? (int)BUF_B : (int)BUF_A;
+        };
+        PassPlan pl;
+        pl.active = (active >> t) & 1u;
+        pl.src = idx == 0 ? (int)BUF_USER : target(idx - 1);
+        pl.dst = target(idx);
+        pl.narrow = idx == lw && idx < m - 1;
+        h->plan[t] = pl;
+        if (t == 0) h->identity = m == 0;
     }
 }
 
