@@ -635,7 +635,7 @@ struct SmallItems {
 
 template <typename K>
 struct SmallShared {
-    SmallItems<K> in, staged;    // written by the whole cluster, and by the block
+    SmallItems<K> buf[2];               // the block's positions, written by the whole cluster, and its staged items
     uint32_t wofs[SMALL_WARPS][RADIX];  // per-warp digit counts, then first staged slots
     uint32_t part[4][RADIX];            // digit counts of eight warps each
     uint32_t count[2][RADIX];           // ... and of the block, read by the others (by pass parity)
@@ -676,7 +676,9 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
     const K mask = key_mask<K>(key_bits);
     const uint32_t d = tid & (RADIX - 1), quarter = tid >> 8;
     wait_for_previous();
-    const uint32_t in_key = (uint32_t)__cvta_generic_to_shared(sh.in.key), in_id = (uint32_t)__cvta_generic_to_shared(sh.in.id);
+    const uint32_t in_key = (uint32_t)__cvta_generic_to_shared(sh.buf[0].key);
+    const uint32_t in_id = (uint32_t)__cvta_generic_to_shared(sh.buf[0].id);
+    uint32_t cur = 0;  // the buffer that holds the block's positions; a block alone alternates
     for (uint32_t pass = 0; 8 * pass < key_bits; ++pass) {
         K kreg[SMALL_ITEMS];
         uint32_t vreg[SMALL_ITEMS];
@@ -691,9 +693,9 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
                 kreg[i] = ok ? (K)(keys[first + pos] & mask) : (K)0;
                 vreg[i] = first + pos;
             } else {
-                const uint64_t e = ok ? sh.in.key[pos] : 0ull;
+                const uint64_t e = ok ? sh.buf[cur].key[pos] : 0ull;
                 kreg[i] = (K)e;
-                vreg[i] = PAIRS ? (uint32_t)(e >> 32) : ok ? sh.in.id[pos] : 0u;
+                vreg[i] = PAIRS ? (uint32_t)(e >> 32) : ok ? sh.buf[cur].id[pos] : 0u;
             }
         }
         __syncthreads();  // counts cleared
@@ -715,7 +717,7 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
             total = sh.part[0][d] + sh.part[1][d] + sh.part[2][d] + sh.part[3][d];
             sh.count[pass & 1][d] = total;
         }
-        cluster_arrive();  // this block's counts are written, and its items in registers
+        if (blocks > 1) cluster_arrive();  // this block's counts are written, and its items in registers
         const uint32_t local = digit_scan(total, sh.wsum[0]);
         if (tid < RADIX) sh.start[d] = local;
         __syncthreads();
@@ -728,9 +730,14 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
         for (int i = 0; i < SMALL_ITEMS; ++i) {
             if (wfirst + (uint32_t)i * 32 < tile_n) {
                 const uint32_t slot = sh.wofs[warp][digit_of(kreg[i], pass)] + rank[i];
-                sh.staged.key[slot] = PAIRS ? (uint64_t)vreg[i] << 32 | (uint32_t)kreg[i] : (uint64_t)kreg[i];
-                if (!PAIRS) sh.staged.id[slot] = vreg[i];
+                sh.buf[cur ^ 1].key[slot] = PAIRS ? (uint64_t)vreg[i] << 32 | (uint32_t)kreg[i] : (uint64_t)kreg[i];
+                if (!PAIRS) sh.buf[cur ^ 1].id[slot] = vreg[i];
             }
+        }
+        if (blocks == 1) {  // staged is sorted: no exchange, and the next pass reads it there
+            cur ^= 1;
+            __syncthreads();
+            continue;
         }
         cluster_wait();  // every block's counts
         uint32_t all = 0, before = 0;
@@ -750,20 +757,20 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
         for (int i = 0; i < SMALL_ITEMS; ++i) {
             const uint32_t p = tid + (uint32_t)i * SMALL_BLOCK;
             if (p < tile_n) {
-                const uint64_t e = sh.staged.key[p];
+                const uint64_t e = sh.buf[1].key[p];
                 const uint32_t pos = sh.start[digit_of((K)e, pass)] + p;
                 const uint32_t to = pos / SMALL_CAP, slot = pos % SMALL_CAP;
                 asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_address(in_key + slot * 8u, to)), "l"(e) : "memory");
                 if (!PAIRS)
                     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_address(in_id + slot * 4u, to)),
-                                 "r"(sh.staged.id[p]) : "memory");
+                                 "r"(sh.buf[1].id[p]) : "memory");
             }
         }
         cluster_arrive();
         cluster_wait();  // every item at its place; no block leaves while others may write to it
     }
     for (uint32_t p = tid; p < tile_n; p += SMALL_BLOCK)
-        perm[first + p] = PAIRS ? (uint32_t)(sh.in.key[p] >> 32) : sh.in.id[p];
+        perm[first + p] = PAIRS ? (uint32_t)(sh.buf[cur].key[p] >> 32) : sh.buf[cur].id[p];
 }
 
 template <typename K>
