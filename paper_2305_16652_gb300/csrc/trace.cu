@@ -801,12 +801,13 @@ __device__ __forceinline__ bool start_ray(const TraceArgs &a, uint64_t i, State 
         d4 = __ldcs(a.dir + src * a.rs);
     }
     const SceneDesc *sc = MULTI ? a.scenes + scene_of(a.offsets, a.num_scenes, src) : nullptr;
-    tris = MULTI ? sc->tris : a.tris;
+    if (MULTI) {
+        tris = sc->tris;
+        nodes = LAYOUT == COMPACT ? sc->cnodes : sc->nodes;
+    }
     if constexpr (LAYOUT == COMPACT) {
-        nodes = MULTI ? sc->cnodes : a.cnodes;
         ray_init(s, stack, o4, d4, MULTI ? sc->grid : a.grid, MULTI ? sc->croot : a.croot);
     } else {
-        nodes = MULTI ? sc->nodes : a.nodes;
         ray_init(s, o4, d4, MULTI ? sc->root_ref : a.root_ref);
     }
     return true;
@@ -841,8 +842,8 @@ __device__ __forceinline__ void store_hit(const TraceArgs &a, uint64_t i, const 
 template <bool ANY, bool COUNT, int LAYOUT, bool MULTI>
 __global__ void __launch_bounds__(TRACE_BLOCK, LAYOUT == COMPACT ? 9 : 1) k_trace(TraceArgs a) {
     uint64_t i = (uint64_t)blockIdx.x * TRACE_BLOCK + threadIdx.x;
-    const uint4 *nodes;
-    const float4 *tris;
+    const uint4 *nodes = MULTI ? nullptr : LAYOUT == COMPACT ? a.cnodes : a.nodes;
+    const float4 *tris = MULTI ? nullptr : a.tris;
     StateOf<LAYOUT> s;
     uint2 stack[STACK_SIZE<LAYOUT, STACK>];
     Counters cn;
@@ -904,8 +905,8 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
     uint2 aux[COMPACT_SLOTS], stack[STACK];
     s.node = s.leaf = REF_NONE;
     s.best_prim = -1;
-    const uint4 *nodes;
-    const float4 *tris;
+    const uint4 *nodes = a.cnodes;
+    const float4 *tris = a.tris;
     bool have = i < a.n;
     if (have) {
         if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end, as the other traces
@@ -1049,8 +1050,8 @@ __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
     StateOf<LAYOUT> s;
     uint2 stack[STACK_SIZE<LAYOUT, STACKN>];
     Counters cn;
-    const uint4 *nodes = nullptr;
-    const float4 *tris = nullptr;
+    const uint4 *nodes = MULTI ? nullptr : LAYOUT == COMPACT ? a.cnodes : a.nodes;
+    const float4 *tris = MULTI ? nullptr : a.tris;
     uint32_t slot = 0;  // below n, which fits 32 bits
     bool have = false, exhausted = false;
     const uint32_t stack_base = LAYOUT == COMPACT ? local_address(stack + COMPACT_SLOTS) : 0u;
