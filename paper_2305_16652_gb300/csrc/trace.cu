@@ -614,10 +614,12 @@ __device__ __forceinline__ void pop_node(CompactState &s, uint32_t stack_base) {
         : "+r"(s.node), "+r"(s.sp), "+r"(s.top_ref), "+f"(s.top_t) : "f"(s.tcap), "r"(stack_base) : "memory");
 }
 
-// Entry and exit distance of a child (slab words wx, wy, wz).  The near and far
+// Entry and exit distance of a child (slab words wx, wy, wz); CAP: the exit no later
+// than the best hit.  The near and far
 // bound of an axis come out of its word by byte permutes whose selectors hold the
 // direction's sign, so decoding costs no more than sorting the two distances by
 // min and max would.
+template <bool CAP>
 __device__ __forceinline__ void compact_child(const CompactState &s, uint32_t wx, uint32_t wy, uint32_t wz, float &tn,
                                               float &tf) {
     const float2 n = __ffma2_rn(make_float2(grid_bound(wx, s.sx), grid_bound(wy, s.sy)), s.ixy, s.cxy);
@@ -626,21 +628,31 @@ __device__ __forceinline__ void compact_child(const CompactState &s, uint32_t wx
     const float nz = __saturatef(__fmaf_rn(grid_bound(wz, s.sz), s.iz, s.cz));
     const float fz = __fmaf_rn(grid_bound(wz, s.sz ^ GRID_HI_LO), s.iz, s.cz);
     tn = fmax3(n.x, n.y, nz);
-    tf = fminf(__fadd_rn(fmin3(f.x, f.y, fz), s.widen), s.tcap);
+    tf = __fadd_rn(fmin3(f.x, f.y, fz), s.widen);
+    if (CAP) tf = fminf(tf, s.tcap);
 }
 
-// Pushes a subtree met at distance t (+inf: not met).  TOP: the last push of a
+// Entry distance of a child for the order of a step: its own if the ray meets it,
+// beyond any cap if it does not, by two multiply-adds where a compare and a
+// select would take the ALU pipe.  (A box missed by less than 1e-37 of the scene
+// may count as met, which costs a visit.)
+constexpr float CAP_MAX = 8.0f;  // no box of the scene is met beyond 1
+__device__ __forceinline__ float met_distance(float tn, float tf) {
+    return __fmaf_rn(__saturatef(__fsub_rn(tn, tf)), 1e38f, tn);
+}
+
+// Pushes a subtree met at distance t before the best hit.  TOP: the last push of a
 // step, which leaves the topmost entry.
 template <bool TOP>
 __device__ __forceinline__ void push_node(CompactState &s, uint32_t ref, float t) {
     if (TOP)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %4, 0f7F800000;\n\t"
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %4, %5;\n\t"
             "@p st.local.v2.b32 [%0], {%3, %4};\n\t@p add.u32 %0, %0, 8;\n\t@p mov.b32 %1, %3;\n\t@p mov.b32 %2, %4;\n\t}"
-            : "+r"(s.sp), "+r"(s.top_ref), "+f"(s.top_t) : "r"(ref), "f"(t) : "memory");
+            : "+r"(s.sp), "+r"(s.top_ref), "+f"(s.top_t) : "r"(ref), "f"(t), "f"(s.tcap) : "memory");
     else
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %2, 0f7F800000;\n\t"
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %2, %3;\n\t"
             "@p st.local.v2.b32 [%0], {%1, %2};\n\t@p add.u32 %0, %0, 8;\n\t}"
-            : "+r"(s.sp) : "r"(ref), "f"(t) : "memory");
+            : "+r"(s.sp) : "r"(ref), "f"(t), "f"(s.tcap) : "memory");
 }
 
 // One node step: tests the four children, descends into the nearest one met
@@ -653,10 +665,10 @@ __device__ __forceinline__ void node_step(CompactState &s, const uint4 *__restri
     ldg256(nodes + 4 * (size_t)s.node, w0, w1);
     ldg256(nodes + 4 * (size_t)s.node + 2, w2, rf);
     float n0, n1, n2, n3, f0, f1, f2, f3;
-    compact_child(s, w0.x, w0.y, w0.z, n0, f0);
-    compact_child(s, w0.w, w1.x, w1.y, n1, f1);
-    compact_child(s, w1.z, w1.w, w2.x, n2, f2);
-    compact_child(s, w2.y, w2.z, w2.w, n3, f3);
+    compact_child<ANY>(s, w0.x, w0.y, w0.z, n0, f0);
+    compact_child<ANY>(s, w0.w, w1.x, w1.y, n1, f1);
+    compact_child<ANY>(s, w1.z, w1.w, w2.x, n2, f2);
+    compact_child<ANY>(s, w2.y, w2.z, w2.w, n3, f3);
     if (ANY) {
         // no order and no distance: every met child is pushed, the last taken back
         asm volatile("{\n\t.reg .pred h0, h1, h2, h3, p;\n\t"
@@ -672,18 +684,17 @@ __device__ __forceinline__ void node_step(CompactState &s, const uint4 *__restri
             : "memory");
         return;
     }
-    const float INF = __int_as_float(0x7F800000);
-    n0 = n0 < f0 ? n0 : INF;
-    n1 = n1 < f1 ? n1 : INF;
-    n2 = n2 < f2 ? n2 : INF;
-    n3 = n3 < f3 ? n3 : INF;
+    n0 = met_distance(n0, f0);
+    n1 = met_distance(n1, f1);
+    n2 = met_distance(n2, f2);
+    n3 = met_distance(n3, f3);
     uint32_t r0 = rf.x, r1 = rf.y, r2 = rf.z, r3 = rf.w;
     order2(n0, r0, n1, r1);
     order2(n2, r2, n3, r3);
     order2(n0, r0, n2, r2);
     order2(n1, r1, n3, r3);
     order2(n1, r1, n2, r2);
-    s.node = n0 < INF ? r0 : REF_NONE;
+    s.node = n0 < s.tcap ? r0 : REF_NONE;
     push_node<false>(s, r3, n3);
     push_node<false>(s, r2, n2);
     push_node<true>(s, r1, n1);
@@ -780,7 +791,7 @@ __device__ __forceinline__ void add_counts(const TraceArgs &a, const Counters &c
 
 // Reads ray slot i (the ray is org/dir[gather[i]], or i) and sets up its
 // traversal.  Returns false (and reports) for an out-of-range permutation entry.
-template <bool MULTI, int LAYOUT, typename State>
+template <bool ANY, bool MULTI, int LAYOUT, typename State>
 __device__ __forceinline__ bool start_ray(const TraceArgs &a, uint64_t i, State &s, uint2 *stack,
                                           const uint4 *&nodes, const float4 *&tris) {
     float4 o4, d4;
@@ -807,6 +818,7 @@ __device__ __forceinline__ bool start_ray(const TraceArgs &a, uint64_t i, State 
     }
     if constexpr (LAYOUT == COMPACT) {
         ray_init(s, stack, o4, d4, MULTI ? sc->grid : a.grid, MULTI ? sc->croot : a.croot);
+        if (!ANY) s.tcap = fminf(s.tcap, CAP_MAX);
     } else {
         ray_init(s, o4, d4, MULTI ? sc->root_ref : a.root_ref);
     }
@@ -850,7 +862,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, LAYOUT == COMPACT ? 9 : 1) k_trac
     bool have = i < a.n;
     if (have) {
         if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end (blocks start in index order)
-        have = start_ray<MULTI, LAYOUT>(a, i, s, stack, nodes, tris);
+        have = start_ray<ANY, MULTI, LAYOUT>(a, i, s, stack, nodes, tris);
     }
     if constexpr (LAYOUT == COMPACT) {
         const uint32_t base = local_address(stack + COMPACT_SLOTS);
@@ -910,7 +922,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
     bool have = i < a.n;
     if (have) {
         if (a.gather || a.scatter) i = a.n - 1 - i;  // sorted order from its end, as the other traces
-        have = start_ray<false, COMPACT>(a, i, s, aux, nodes, tris);
+        have = start_ray<ANY, false, COMPACT>(a, i, s, aux, nodes, tris);
     }
     const float tmin = __uint_as_float(aux[0].x), scale = __uint_as_float(aux[0].y), from = __uint_as_float(aux[1].x);
     uint32_t level = 1;  // of the current node's children
@@ -941,7 +953,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
                 const uint32_t wx = __ldg(w + 3 * child), wy = __ldg(w + 3 * child + 1), wz = __ldg(w + 3 * child + 2);
                 ref = __ldg(w + 12 + child);
                 float tn, tf;
-                compact_child(s, wx, wy, wz, tn, tf);
+                compact_child<true>(s, wx, wy, wz, tn, tf);
                 if (tn < tf) key = ((63u - level) << 24) | ((__float_as_uint(tn) >> 6) & 0x00FFFFFCu) | child;
             }
             const bool met = key != QUAD_NONE;
@@ -1070,7 +1082,7 @@ __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
                 const uint64_t at = base + __popc(need & lt);
                 if (at < a.n) {
                     slot = (uint32_t)((a.gather || a.scatter) ? a.n - 1 - at : at);  // sorted order from its end
-                    have = start_ray<MULTI, LAYOUT>(a, slot, s, stack, nodes, tris);
+                    have = start_ray<ANY, MULTI, LAYOUT>(a, slot, s, stack, nodes, tris);
                 } else {
                     exhausted = true;
                 }
