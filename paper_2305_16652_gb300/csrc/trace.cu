@@ -731,7 +731,6 @@ __device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, u
     bool more;
     do {
         pop_node<ANY>(s, stack_base);
-        park_leaf(s);
         if ((int)s.node >= 0) node_step<ANY>(s, nodes);
         park_leaf(s);
         more = s.leaf == REF_NONE && (s.node != REF_NONE || s.sp != stack_base);
