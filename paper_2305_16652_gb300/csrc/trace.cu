@@ -442,8 +442,8 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
 // of two that brings the scene's far side below 1: a saturating fma then
 // clamps the entry distance to the ray's start.
 struct CompactState {
-    float2 ixy, cxy;
-    float iz, cz;
+    float2 ixy, cxy, far_cxy;  // far_c: c + widen, rounded up
+    float iz, cz, far_cz;
     uint32_t sx, sy, sz;  // byte selectors of each axis's near bound (lo or hi by the direction's sign)
     float tcap;           // tau of the best hit widened by the prune slack
     float widen;          // added to a box's exit distance (0 unless the origin is far outside the scene)
@@ -562,6 +562,8 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     s.sz = iz < 0.0f ? 0x4325u : 0x4105u;
     s.tcap = __fmul_ru(tmax, scale);
     s.widen = far ? fminf(__fmul_rn(__fmul_rn(fabsf(from), FAR_WIDEN), scale), FAR_WIDEN_MAX) : 0.0f;
+    s.far_cxy = make_float2(__fadd_ru(s.cxy.x, s.widen), __fadd_ru(s.cxy.y, s.widen));
+    s.far_cz = __fadd_ru(s.cz, s.widen);
     s.best_t = d4.w;
     s.best_u = s.best_v = 0.0f;
     s.best_prim = -1;
@@ -615,20 +617,21 @@ __device__ __forceinline__ void pop_node(CompactState &s, uint32_t stack_base) {
 }
 
 // Entry and exit distance of a child (slab words wx, wy, wz); CAP: the exit no later
-// than the best hit.  The near and far
+// than the best hit; FAR_C: the exit widened by its own constants.  The near and far
 // bound of an axis come out of its word by byte permutes whose selectors hold the
 // direction's sign, so decoding costs no more than sorting the two distances by
 // min and max would.
-template <bool CAP>
+template <bool CAP, bool FAR_C>
 __device__ __forceinline__ void compact_child(const CompactState &s, uint32_t wx, uint32_t wy, uint32_t wz, float &tn,
                                               float &tf) {
     const float2 n = __ffma2_rn(make_float2(grid_bound(wx, s.sx), grid_bound(wy, s.sy)), s.ixy, s.cxy);
     const float2 f = __ffma2_rn(make_float2(grid_bound(wx, s.sx ^ GRID_HI_LO), grid_bound(wy, s.sy ^ GRID_HI_LO)),
-                                s.ixy, s.cxy);
+                                s.ixy, FAR_C ? s.far_cxy : s.cxy);
     const float nz = __saturatef(__fmaf_rn(grid_bound(wz, s.sz), s.iz, s.cz));
-    const float fz = __fmaf_rn(grid_bound(wz, s.sz ^ GRID_HI_LO), s.iz, s.cz);
+    const float fz = __fmaf_rn(grid_bound(wz, s.sz ^ GRID_HI_LO), s.iz, FAR_C ? s.far_cz : s.cz);
     tn = fmax3(n.x, n.y, nz);
-    tf = __fadd_rn(fmin3(f.x, f.y, fz), s.widen);
+    tf = fmin3(f.x, f.y, fz);
+    if (!FAR_C) tf = __fadd_rn(tf, s.widen);
     if (CAP) tf = fminf(tf, s.tcap);
 }
 
@@ -659,16 +662,20 @@ __device__ __forceinline__ void push_node(CompactState &s, uint32_t ref, float t
 // and pushes the others, farthest first.  (Pushing them unsorted saved 10
 // instructions of 185 a step but took 13 % more steps; multiply-adds in place of
 // the selects of the exchanges, to relieve the ALU pipe, changed nothing.)
-template <bool ANY>
+// FAR_C pays where three registers are left for it: an addition per child less
+// for single wavefronts' closest hits (1080p bounce 3736 -> 3674 us, 2.1M unsorted 409 ->
+// 400), but any hit (559 -> 566 us for 4.1M shadow rays) and a batch (1188 -> 1230)
+// run out of registers.
+template <bool ANY, bool FAR_C>
 __device__ __forceinline__ void node_step(CompactState &s, const uint4 *__restrict__ nodes) {
     uint4 w0, w1, w2, rf;
     ldg256(nodes + 4 * (size_t)s.node, w0, w1);
     ldg256(nodes + 4 * (size_t)s.node + 2, w2, rf);
     float n0, n1, n2, n3, f0, f1, f2, f3;
-    compact_child<ANY>(s, w0.x, w0.y, w0.z, n0, f0);
-    compact_child<ANY>(s, w0.w, w1.x, w1.y, n1, f1);
-    compact_child<ANY>(s, w1.z, w1.w, w2.x, n2, f2);
-    compact_child<ANY>(s, w2.y, w2.z, w2.w, n3, f3);
+    compact_child<ANY, FAR_C>(s, w0.x, w0.y, w0.z, n0, f0);
+    compact_child<ANY, FAR_C>(s, w0.w, w1.x, w1.y, n1, f1);
+    compact_child<ANY, FAR_C>(s, w1.z, w1.w, w2.x, n2, f2);
+    compact_child<ANY, FAR_C>(s, w2.y, w2.z, w2.w, n3, f3);
     if (ANY) {
         // no order and no distance: every met child is pushed, the last taken back
         asm volatile("{\n\t.reg .pred h0, h1, h2, h3, p;\n\t"
@@ -724,14 +731,14 @@ __device__ __forceinline__ float4 ldg_first(const float4 *p) {
 // their order against 596 with a slack of 4 lanes.)
 constexpr int COMPACT_SLACK = 6;    // 3: 1.5 % slower in HCC order, 5 % unsorted; 10: equal
 constexpr int COMPACT_TRI_MIN = 6;  // 4 and 8 within 0.5 %
-template <bool ANY>
+template <bool ANY, bool FAR_C>
 __device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, uint32_t stack_base,
                                           const uint4 *__restrict__ nodes, const float4 *__restrict__ tris) {
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     bool more;
     do {
         pop_node<ANY>(s, stack_base);
-        if ((int)s.node >= 0) node_step<ANY>(s, nodes);
+        if ((int)s.node >= 0) node_step<ANY, FAR_C>(s, nodes);
         park_leaf(s);
         more = s.leaf == REF_NONE && (s.node != REF_NONE || s.sp != stack_base);
     } while (__popc(__ballot_sync(FULL, more)) > (ANY ? 0 : COMPACT_SLACK));
@@ -867,7 +874,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, LAYOUT == COMPACT ? 9 : 1) k_trac
         const uint32_t base = local_address(stack + COMPACT_SLOTS);
         s.sp = base;
         if (!have) ray_none(s, base);
-        while (__any_sync(0xFFFFFFFFu, !ray_done(s, base))) ray_round<ANY>(s, stack, base, nodes, tris);
+        while (__any_sync(0xFFFFFFFFu, !ray_done(s, base))) ray_round<ANY, false>(s, stack, base, nodes, tris);
         if (!have) return;
     } else {
         if (!have) return;
@@ -952,7 +959,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK) k_trace_quad(TraceArgs a) {
                 const uint32_t wx = __ldg(w + 3 * child), wy = __ldg(w + 3 * child + 1), wz = __ldg(w + 3 * child + 2);
                 ref = __ldg(w + 12 + child);
                 float tn, tf;
-                compact_child<true>(s, wx, wy, wz, tn, tf);
+                compact_child<true, false>(s, wx, wy, wz, tn, tf);
                 if (tn < tf) key = ((63u - level) << 24) | ((__float_as_uint(tn) >> 6) & 0x00FFFFFCu) | child;
             }
             const bool met = key != QUAD_NONE;
@@ -1093,7 +1100,7 @@ __global__ void __launch_bounds__(BLOCK, pool_threads(LAYOUT, MULTI) / BLOCK)
         }
         bool done;
         if constexpr (LAYOUT == COMPACT) {
-            ray_round<ANY>(s, stack, stack_base, nodes, tris);
+            ray_round<ANY, !ANY && !MULTI>(s, stack, stack_base, nodes, tris);
             done = ray_done(s, stack_base);
         }
         if (have) {
