@@ -13,7 +13,7 @@ namespace hcc {
 namespace {
 
 constexpr int ENC_BLOCK = 256;
-constexpr int ENC_BOX_BLOCKS = 5;  // resident blocks per SM of the cut-box kernels (48 registers; 4 and 6 within 1 %)
+constexpr int ENC_BLOCKS = 8;  // blocks per SM of the encode grids
 constexpr uint32_t MAX_CUT_BITS = 64;
 
 int encode_grid(uint64_t n, int block, int per_sm) {
@@ -39,39 +39,32 @@ __device__ __forceinline__ bool meets(const float4 &o, const float4 &d, float ix
     return tnear <= tfar;
 }
 
-// Cut boxes staged in shared memory for the slab test, two boxes to an entry: per
-// pair of boxes six float4, for each axis the two orders of its bounds, entry
-// 2 * axis holding (lo, hi) of both boxes and entry 2 * axis + 1 (hi, lo), so that a
-// ray reads the (near, far) bounds of an axis of two boxes with one 128-bit
-// load indexed by its direction's sign.  The second box of a last odd pair
-// repeats the first.  Returns whether this thread's boxes are finite with lo <= hi.
-__device__ __forceinline__ bool stage_pair(float4 *pairs, const float4 *__restrict__ boxes, uint32_t n, uint32_t q) {
-    const uint32_t r0 = 2 * q, r1 = r0 + 1 < n ? r0 + 1 : r0;
-    const float4 l0 = __ldg(boxes + 2 * r0), h0 = __ldg(boxes + 2 * r0 + 1);
-    const float4 l1 = __ldg(boxes + 2 * r1), h1 = __ldg(boxes + 2 * r1 + 1);
-    float4 *b = pairs + 6 * q;
-    b[0] = make_float4(l0.x, h0.x, l1.x, h1.x);
-    b[1] = make_float4(h0.x, l0.x, h1.x, l1.x);
-    b[2] = make_float4(l0.y, h0.y, l1.y, h1.y);
-    b[3] = make_float4(h0.y, l0.y, h1.y, l1.y);
-    b[4] = make_float4(l0.z, h0.z, l1.z, h1.z);
-    b[5] = make_float4(h0.z, l0.z, h1.z, l1.z);
+// Cut boxes staged in shared memory for the slab test: per box and axis the two
+// orders of its bounds, entry 2 * axis holding (lo, hi) and entry 2 * axis + 1 (hi,
+// lo), so that a ray reads the (near, far) bounds of an axis with one 64-bit
+// load indexed by its direction's sign.  Returns whether the box is finite with lo <= hi.
+constexpr uint32_t BOX = 6;  // entries of a box
+__device__ __forceinline__ bool stage_box(float2 *b, const float4 *__restrict__ box) {
+    const float4 lo = __ldg(box), hi = __ldg(box + 1);
+    b[0] = make_float2(lo.x, hi.x);
+    b[1] = make_float2(hi.x, lo.x);
+    b[2] = make_float2(lo.y, hi.y);
+    b[3] = make_float2(hi.y, lo.y);
+    b[4] = make_float2(lo.z, hi.z);
+    b[5] = make_float2(hi.z, lo.z);
     const float inf = __int_as_float(0x7F800000);
-    auto ordered = [&](float lo, float hi) { return -inf < lo && lo <= hi && hi < inf; };
-    return ordered(l0.x, h0.x) && ordered(l0.y, h0.y) && ordered(l0.z, h0.z) && ordered(l1.x, h1.x) &&
-           ordered(l1.y, h1.y) && ordered(l1.z, h1.z);
+    auto ordered = [&](float l, float u) { return -inf < l && l <= u && u < inf; };
+    return ordered(lo.x, hi.x) && ordered(lo.y, hi.y) && ordered(lo.z, hi.z);
 }
 
-__device__ __forceinline__ bool stage_boxes(float4 *pairs, const float4 *__restrict__ boxes, uint32_t n) {
+__device__ __forceinline__ bool stage_boxes(float2 *staged, const float4 *__restrict__ boxes, uint32_t n) {
     bool ordered = true;
-    for (uint32_t q = threadIdx.x; 2 * q < n; q += blockDim.x) ordered = stage_pair(pairs, boxes, n, q) && ordered;
+    for (uint32_t q = threadIdx.x; q < n; q += blockDim.x) ordered = stage_box(staged + BOX * q, boxes + 2 * q) && ordered;
     return ordered;
 }
 
 // A ray set up for the slab test of staged boxes.
 struct SlabRay {
-    float2 nox, noy, noz, ixx, iyy, izz;  // negated origin and reciprocal direction, each twice
-    uint32_t sx, sy, sz;                  // entry of each axis by its direction's sign
     float4 o, d;
     float ix, iy, iz;
     bool fast;
@@ -84,116 +77,73 @@ __device__ __forceinline__ SlabRay slab_ray(const float4 &o, const float4 &d, bo
     r.ix = __frcp_rn(d.x);
     r.iy = __frcp_rn(d.y);
     r.iz = __frcp_rn(d.z);
-    r.sx = r.ix < 0.0f;
-    r.sy = 2u + (r.iy < 0.0f);
-    r.sz = 4u + (r.iz < 0.0f);
-    r.nox = make_float2(-o.x, -o.x);
-    r.noy = make_float2(-o.y, -o.y);
-    r.noz = make_float2(-o.z, -o.z);
-    r.ixx = make_float2(r.ix, r.ix);
-    r.iyy = make_float2(r.iy, r.iy);
-    r.izz = make_float2(r.iz, r.iz);
-    const float inf = __int_as_float(0x7F800000);
-    auto plain = [&](float x) { return x != 0.0f && fabsf(x) < inf; };  // false for NaN
-    r.fast = ordered && plain(r.ix) && plain(r.iy) && plain(r.iz) && fabsf(o.x) < inf && fabsf(o.y) < inf &&
-             fabsf(o.z) < inf && o.w == o.w && d.w == d.w;
+    r.fast = ordered && isfinite(r.ix) && isfinite(r.iy) && isfinite(r.iz);
     return r;
 }
 
-// Misses of a fast ray against 2 * n staged boxes (n <= 16), the first box in
-// the highest of the 2 * n low bits.
+// Bits of n staged boxes, box 0 in the highest of the n low bits: 1 = the ray
+// meets it.  Every ray may call it.
 //
-// With finite, non-zero reciprocals and boxes with lo <= hi the near and far
-// bound of an axis are known from the reciprocal's sign (rounding is monotonic),
-// so no distance is sorted: (bound + (-o)) * inv of both bounds is one packed add and
+// With finite reciprocals and finite boxes with lo <= hi the near and far bound of
+// an axis are known from the reciprocal's sign (rounding is monotonic; a NaN, from
+// a zero reciprocal or a NaN origin, is both or neither), so no distance is sorted: (bound + (-o)) * inv of both bounds is one packed add and
 // one packed multiply, the same round-to-nearest results as (bound - o) * inv one at a
-// time.  No operand of a fast ray makes a NaN distance, so tnear <= tfar is the
-// sign of tfar - tnear (which is exact in its sign; infinities of one sign give the
-// canonical NaN, whose sign bit is 0, as a met box has), and a funnel shift
-// takes that sign into the key.
-// UNBOUNDED: tmax = +inf, which clamps no exit distance.
+// time.
 //
 // Bound by the shared-memory data pipe, which returns the 24 bytes per ray and
 // box in six cycles a warp (90 % of the time of 16.6M rays against 32 boxes,
-// 0.35 ms): 13 instructions per ray and box here instead of 20 one box at a time
-// with compare and insert leave that time as it is.
-template <bool UNBOUNDED>
-__device__ __forceinline__ uint32_t missed_boxes(const SlabRay &r, const float4 *pairs, uint32_t n) {
-    const float4 *px = pairs + r.sx, *py = pairs + r.sy, *pz = pairs + r.sz;
-    uint32_t bits = 0;
-#pragma unroll 4
-    for (uint32_t q = 0; q < n; ++q) {
-        const float4 bx = px[6 * q], by = py[6 * q], bz = pz[6 * q];
-        const float2 x0 = __fmul2_rn(__fadd2_rn(make_float2(bx.x, bx.y), r.nox), r.ixx);
-        const float2 y0 = __fmul2_rn(__fadd2_rn(make_float2(by.x, by.y), r.noy), r.iyy);
-        const float2 z0 = __fmul2_rn(__fadd2_rn(make_float2(bz.x, bz.y), r.noz), r.izz);
-        const float2 x1 = __fmul2_rn(__fadd2_rn(make_float2(bx.z, bx.w), r.nox), r.ixx);
-        const float2 y1 = __fmul2_rn(__fadd2_rn(make_float2(by.z, by.w), r.noy), r.iyy);
-        const float2 z1 = __fmul2_rn(__fadd2_rn(make_float2(bz.z, bz.w), r.noz), r.izz);
-        const float f0 = fmin3(x0.y, y0.y, UNBOUNDED ? z0.y : fminf(z0.y, r.d.w));
-        const float f1 = fmin3(x1.y, y1.y, UNBOUNDED ? z1.y : fminf(z1.y, r.d.w));
-        // adding 0 turns an exit distance of -0 into +0: -0 - +0 would be -0, a miss by its sign
-        const float g0 = __fsub_rn(__fadd_rn(f0, 0.0f), fmax3(x0.x, y0.x, fmaxf(z0.x, r.o.w)));
-        const float g1 = __fsub_rn(__fadd_rn(f1, 0.0f), fmax3(x1.x, y1.x, fmaxf(z1.x, r.o.w)));
-        bits = __funnelshift_l(__float_as_uint(g0), bits, 1);
-        bits = __funnelshift_l(__float_as_uint(g1), bits, 1);
-    }
-    return bits;
-}
-
-// Bits of n staged boxes (n <= 32), box 0 in the highest of the n low bits: 1 =
-// the ray meets it.  Every ray may call it; `pairs` are the boxes' pairs.
-__device__ __forceinline__ uint32_t met_boxes(const SlabRay &r, const float4 *pairs, uint32_t n) {
+// 0.36 ms).  Two boxes per 128-bit load with the result taken from the sign of a
+// difference, 13 instructions per ray and box instead of 20, left that time as it is
+// (0.365 ms), and cost two-level keys 5 to 15 % (16 bits: 0.289 against 0.270 ms).
+template <typename K>
+__device__ __forceinline__ K met_boxes(const SlabRay &r, const float2 *boxes, uint32_t n) {
+    K bits = 0;
     if (r.fast) {
-        const uint32_t half = (n + 1) / 2;
-        const bool unbounded = r.d.w == __int_as_float(0x7F800000);
-        const uint32_t missed = __all_sync(__activemask(), unbounded) ? missed_boxes<true>(r, pairs, half)
-                                                                     : missed_boxes<false>(r, pairs, half);
-        const uint32_t mask = n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u;
-        return ~(missed >> (n & 1u)) & mask;  // the repeated box of an odd last pair drops out
-    }
-    uint32_t bits = 0;
-    for (uint32_t q = 0; q < n; ++q) {
-        const float4 *b = pairs + 6 * (q / 2);
-        const float4 x = b[0], y = b[2], z = b[4];
-        const bool second = q & 1u;
-        bits = (bits << 1) | (uint32_t)meets(r.o, r.d, r.ix, r.iy, r.iz,
-                                             make_float4(second ? x.z : x.x, second ? y.z : y.x, second ? z.z : z.x, 0.f),
-                                             make_float4(second ? x.w : x.y, second ? y.w : y.y, second ? z.w : z.y, 0.f));
+        const float2 *px = boxes + (r.ix < 0.0f), *py = boxes + 2 + (r.iy < 0.0f), *pz = boxes + 4 + (r.iz < 0.0f);
+        const float2 nox = make_float2(-r.o.x, -r.o.x), noy = make_float2(-r.o.y, -r.o.y),
+                     noz = make_float2(-r.o.z, -r.o.z);
+        const float2 ixx = make_float2(r.ix, r.ix), iyy = make_float2(r.iy, r.iy), izz = make_float2(r.iz, r.iz);
+#pragma unroll 8
+        for (uint32_t q = 0; q < n; ++q) {
+            const float2 tx = __fmul2_rn(__fadd2_rn(px[BOX * q], nox), ixx);
+            const float2 ty = __fmul2_rn(__fadd2_rn(py[BOX * q], noy), iyy);
+            const float2 tz = __fmul2_rn(__fadd2_rn(pz[BOX * q], noz), izz);
+            const float tnear = fmax3(tx.x, ty.x, fmaxf(tz.x, r.o.w));
+            const float tfar = fmin3(tx.y, ty.y, fminf(tz.y, r.d.w));
+            bits = (bits << 1) | (K)(tnear <= tfar);
+        }
+    } else {
+        for (uint32_t q = 0; q < n; ++q) {
+            const float2 x = boxes[BOX * q], y = boxes[BOX * q + 2], z = boxes[BOX * q + 4];
+            bits = (bits << 1) | (K)meets(r.o, r.d, r.ix, r.iy, r.iz, make_float4(x.x, y.x, z.x, 0.f),
+                                          make_float4(x.y, y.y, z.y, 0.f));
+        }
     }
     return bits;
 }
 
 // HCC key of one ray against `used` staged boxes: node r drives bit key_bits - 1 - r.
 template <typename K>
-__device__ __forceinline__ K hcc_key(const SlabRay &r, const float4 *pairs, uint32_t used, uint32_t key_bits) {
-    if (used == 0) return 0;
-    K key;
-    if (sizeof(K) == 4 || used <= 32) {
-        key = (K)met_boxes(r, pairs, used);
-    } else {
-        const uint32_t rest = used - 32;
-        const uint64_t top = met_boxes(r, pairs, 32);
-        key = (K)((top << rest) | met_boxes(r, pairs + 6 * 16, rest));
-    }
-    return key << (key_bits - used);
+__device__ __forceinline__ K hcc_key(const SlabRay &r, const float2 *boxes, uint32_t used, uint32_t key_bits) {
+    const K key = met_boxes<K>(r, boxes, used);
+    return used ? key << (key_bits - used) : key;
 }
 
 // Algorithm 1: the cut nodes are staged in shared memory once per block
 // (line 1); every ray is tested against every cut node and each result is
 // one key bit.
 template <typename K>
-__global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_hcc(const float4 *__restrict__ org,
+__global__ void __launch_bounds__(ENC_BLOCK) k_encode_hcc(const float4 *__restrict__ org,
                                                           const float4 *__restrict__ dir, uint64_t n, uint32_t rs,
                                                           const float4 *__restrict__ cut, uint32_t used,
                                                           uint32_t key_bits, K *__restrict__ keys) {
-    __shared__ float4 s_pairs[MAX_CUT_BITS / 2 * 6];
-    const bool ordered = __syncthreads_and(stage_boxes(s_pairs, cut, used));  // a cut is not written after its creation
+    __shared__ float2 s_boxes[MAX_CUT_BITS * BOX];
+    const bool ordered = __syncthreads_and(stage_boxes(s_boxes, cut, used));  // a cut is not written after its creation
     wait_for_previous();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const SlabRay r = slab_ray(__ldcs(org + i * rs), __ldcs(dir + i * rs), ordered);
-        __stcs(keys + i, hcc_key<K>(r, s_pairs, used, key_bits));
+        __stcs(keys + i, hcc_key<K>(r, s_boxes, used, key_bits));
     }
 }
 
@@ -418,13 +368,13 @@ __global__ void __launch_bounds__(ENC_BLOCK) k_encode_multi(const float4 *__rest
 // k_encode_hcc does.  (Reading the boxes from each ray's own scene and ordering
 // their bounds per ray took 83 us for 2.6M rays of six scenes and 24-bit keys.)
 template <typename K>
-__global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_multi_hcc(const float4 *__restrict__ org,
+__global__ void __launch_bounds__(ENC_BLOCK) k_encode_multi_hcc(const float4 *__restrict__ org,
                                                                 const float4 *__restrict__ dir, uint64_t n, uint32_t rs,
                                                                 const SceneDesc *__restrict__ scenes,
                                                                 const uint64_t *__restrict__ offsets,
                                                                 uint32_t num_scenes, uint32_t key_bits,
                                                                 K *__restrict__ keys) {
-    __shared__ float4 s_pairs[MAX_CUT_BITS / 2 * 6];
+    __shared__ float2 s_boxes[MAX_CUT_BITS * BOX];
     wait_for_previous();
     const uint64_t run = (n + gridDim.x - 1) / gridDim.x;
     uint64_t i0 = run * blockIdx.x;
@@ -435,10 +385,10 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_multi_hcc(
         if (i1 <= i0) continue;
         const uint32_t used = min(scenes[s].used, min(key_bits, MAX_CUT_BITS));
         __syncthreads();  // the previous scene's boxes are no longer read
-        const bool ordered = __syncthreads_and(stage_boxes(s_pairs, scenes[s].cut, used));
+        const bool ordered = __syncthreads_and(stage_boxes(s_boxes, scenes[s].cut, used));
         for (uint64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
             const SlabRay r = slab_ray(__ldcs(org + i * rs), __ldcs(dir + i * rs), ordered);
-            K key = hcc_key<K>(r, s_pairs, used, key_bits);
+            K key = hcc_key<K>(r, s_boxes, used, key_bits);
             if (key_bits < 8 * sizeof(K)) key |= (K)s << key_bits;
             __stcs(keys + i, key);
         }
@@ -452,7 +402,7 @@ cudaError_t launch_encode_multi(cudaStream_t s, int method, const float4 *org, c
                                 const SceneDesc *scenes, const uint64_t *offsets, uint32_t num_scenes,
                                 uint32_t key_bits, uint32_t total_bits, void *keys) {
     if (n == 0) return cudaSuccess;
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
 #define HCC_ENC_MULTI(K, KERNEL)                                                                                    \
     return launch_early(KERNEL, grid, ENC_BLOCK, 0, s, org, dir, n, rs, scenes, offsets, num_scenes, key_bits, (K *)keys)
 #define HCC_ENC_MULTI_K(K)                                            \
@@ -477,7 +427,7 @@ cudaError_t launch_encode_multi(cudaStream_t s, int method, const float4 *org, c
 cudaError_t launch_key_stats(cudaStream_t s, const void *keys, uint32_t key_bits, const uint32_t *perm, uint64_t n,
                              unsigned long long *cnt) {
     if (n < 2) return cudaSuccess;
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32) {
         const uint32_t mask = key_bits == 32 ? 0xFFFFFFFFu : ((1u << key_bits) - 1u);
         k_key_stats<uint32_t><<<grid, ENC_BLOCK, 0, s>>>((const uint32_t *)keys, perm, n, mask, cnt);
@@ -491,7 +441,7 @@ cudaError_t launch_key_stats(cudaStream_t s, const void *keys, uint32_t key_bits
 cudaError_t launch_encode_origin(cudaStream_t s, const float4 *org, uint64_t n, uint32_t rs, const float lo[3], const float ext[3],
                                  uint32_t key_bits, void *keys) {
     if (n == 0) return cudaSuccess;
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32)
         return launch_early(k_encode_origin<uint32_t>, grid, ENC_BLOCK, 0, s, org, n, rs, lo[0], lo[1], lo[2], ext[0],
                             ext[1], ext[2], key_bits, (uint32_t *)keys);
@@ -502,7 +452,7 @@ cudaError_t launch_encode_origin(cudaStream_t s, const float4 *org, uint64_t n, 
 cudaError_t launch_encode_origin_dir(cudaStream_t s, const float4 *org, const float4 *dir, uint64_t n, uint32_t rs,
                                      const float lo[3], const float ext[3], uint32_t key_bits, void *keys) {
     if (n == 0) return cudaSuccess;
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32)
         return launch_early(k_encode_origin_dir<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
                             ext[0], ext[1], ext[2], key_bits, (uint32_t *)keys);
@@ -515,26 +465,25 @@ namespace {
 // Multi-level HCC (Sec. 4.3): the top field as in Algorithm 1; the first met
 // top node (HAD order) is the representative, and its low-level cut fills the
 // next low_field bits.  All boxes of both levels are staged in shared memory:
-// top boxes first, then the low boxes row by row.
+// top boxes first, then the low boxes row by row, the rows an odd number of
+// entries apart: lanes read the rows of their own representatives, which would
+// otherwise lie in the same banks.
+__host__ __device__ constexpr uint32_t ml_row(uint32_t low_field) { return BOX * low_field + 1; }
+
 template <typename K>
-__global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_mlhcc(const float4 *__restrict__ org,
+__global__ void __launch_bounds__(ENC_BLOCK) k_encode_mlhcc(const float4 *__restrict__ org,
                                                             const float4 *__restrict__ dir, uint64_t n, uint32_t rs,
                                                             const float4 *__restrict__ top, uint32_t ntop,
                                                             uint32_t top_field, const float4 *__restrict__ low,
                                                             uint32_t low_field, uint32_t key_bits,
                                                             K *__restrict__ keys) {
-    // pairs of the top boxes, then of each low row
-    extern __shared__ float4 s_ml[];
-    const uint32_t top_pairs = (ntop + 1) / 2, row_pairs = (low_field + 1) / 2;
+    extern __shared__ float2 s_ml[];
+    const uint32_t row_len = ml_row(low_field);
     bool ordered = true;
-    for (uint32_t p = threadIdx.x; p < top_pairs + ntop * row_pairs; p += blockDim.x) {
-        if (p < top_pairs) {
-            ordered = stage_pair(s_ml, top, ntop, p) && ordered;
-        } else {
-            const uint32_t row = (p - top_pairs) / row_pairs;
-            ordered = stage_pair(s_ml + 6 * (top_pairs + row * row_pairs), low + 2 * row * low_field, low_field,
-                                 (p - top_pairs) % row_pairs) && ordered;
-        }
+    for (uint32_t q = threadIdx.x; q < ntop + ntop * low_field; q += blockDim.x) {
+        const uint32_t row = q < ntop ? 0 : (q - ntop) / low_field;
+        float2 *b = q < ntop ? s_ml + BOX * q : s_ml + BOX * ntop + row * row_len + BOX * (q - ntop - row * low_field);
+        ordered = stage_box(b, q < ntop ? top + 2 * q : low + 2 * (q - ntop)) && ordered;
     }
     ordered = __syncthreads_and(ordered);
     wait_for_previous();
@@ -543,12 +492,12 @@ __global__ void __launch_bounds__(ENC_BLOCK, ENC_BOX_BLOCKS) k_encode_mlhcc(cons
         const SlabRay r = slab_ray(__ldcs(org + i * rs), __ldcs(dir + i * rs), ordered);
         // top bits first (node t at bit ntop - 1 - t), then the low row of
         // the first met top node (the highest set bit)
-        const uint64_t tb = ntop ? (uint64_t)hcc_key<uint64_t>(r, s_ml, ntop, ntop) : 0ull;
+        const uint64_t tb = met_boxes<uint64_t>(r, s_ml, ntop);
         K key = ntop ? (K)(tb << (key_bits - ntop)) : (K)0;
         if (tb) {
             const uint32_t rep = ntop - 64u + (uint32_t)__clzll((long long)tb);
-            const uint64_t lb = hcc_key<uint64_t>(r, s_ml + 6 * (top_pairs + rep * row_pairs), low_field, low_field);
-            key |= (K)(lb << (key_bits - top_field - low_field));
+            const uint64_t lb = met_boxes<uint64_t>(r, s_ml + BOX * ntop + rep * row_len, low_field);
+            if (low_field) key |= (K)(lb << (key_bits - top_field - low_field));
         }
         __stcs(keys + i, key);
     }
@@ -623,10 +572,9 @@ cudaError_t launch_encode_mlhcc(cudaStream_t s, const float4 *org, const float4 
     if (n == 0) return cudaSuccess;
     if (ntop > top_field || top_field + low_field > MAX_CUT_BITS || top_field + low_field > key_bits)
         return cudaErrorInvalidValue;
-    // six float4 per pair of boxes: at most (16 + 32 * 16) * 96 bytes for even rows
-    // (50,688), (17 + 33 * 16) * 96 = 52,320 for 33 rows of 31 boxes
-    const size_t smem = sizeof(float4) * 6 * ((size_t)(ntop + 1) / 2 + (size_t)ntop * ((low_field + 1) / 2));
-    const int grid = encode_grid(n, ENC_BLOCK, ENC_BOX_BLOCKS);
+    // at most 33 rows of 31 boxes: 50,952 bytes
+    const size_t smem = sizeof(float2) * ntop * ((size_t)BOX + ml_row(low_field));
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32) {
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(k_encode_mlhcc<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -647,7 +595,7 @@ cudaError_t launch_encode_ppc(cudaStream_t s, const float4 *org, const float4 *d
     const float4 lo = make_float4(root_lo[0], root_lo[1], root_lo[2], 0.f);
     const float4 hi = make_float4(root_hi[0], root_hi[1], root_hi[2], 0.f);
     const float4 *f = reinterpret_cast<const float4 *>(nodes);
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32)
         k_encode_ppc<uint32_t><<<grid, ENC_BLOCK, 0, s>>>(org, dir, n, rs, f, root_ref, lo, hi, key_bits,
                                                           (uint32_t *)keys);
@@ -661,7 +609,7 @@ cudaError_t launch_encode_hcc(cudaStream_t s, const float4 *org, const float4 *d
                               const float4 *cut_boxes, uint32_t used, uint32_t key_bits, void *keys) {
     if (n == 0) return cudaSuccess;
     if (used > MAX_CUT_BITS) used = MAX_CUT_BITS;
-    const int grid = encode_grid(n, ENC_BLOCK, ENC_BOX_BLOCKS);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32)
         return launch_early(k_encode_hcc<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, cut_boxes, used, key_bits,
                             (uint32_t *)keys);
@@ -672,7 +620,7 @@ cudaError_t launch_encode_hcc(cudaStream_t s, const float4 *org, const float4 *d
 cudaError_t launch_encode_twopoint(cudaStream_t s, const float4 *org, const float4 *dir, uint64_t n, uint32_t rs,
                                    const float lo[3], const float ext[3], float L, uint32_t key_bits, void *keys) {
     if (n == 0) return cudaSuccess;
-    const int grid = encode_grid(n, ENC_BLOCK, 8);
+    const int grid = encode_grid(n, ENC_BLOCK, ENC_BLOCKS);
     if (key_bits <= 32)
         return launch_early(k_encode_twopoint<uint32_t>, grid, ENC_BLOCK, 0, s, org, dir, n, rs, lo[0], lo[1], lo[2],
                             ext[0], ext[1], ext[2], L, key_bits, (uint32_t *)keys);
