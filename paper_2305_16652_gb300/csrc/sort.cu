@@ -1,8 +1,9 @@
 // Stable LSD radix sort of ray ids by key (Sec. 4.2.3 "Sorting": keys are
 // sorted as natural numbers; Sec. 5: the sort orders ray indices).
 //
-// Design (one pass per 8-bit digit, "onesweep" structure; up to 65,536 keys
-// k_sort_small does all passes in one launch, in a cluster's shared memory):
+// Design (one pass per 8-bit digit, "onesweep" structure; up to 65,536 32-bit
+// or 4,096 64-bit keys k_sort_small does all passes in one launch, in a cluster's or a
+// block's shared memory):
 //   k_hist   one read of every key builds the digit histograms of all passes
 //            (each warp counts its most common digit in a register, the rest
 //            with shared-memory atomics); the last block to finish scans them
@@ -41,8 +42,9 @@ constexpr int SORT_WARPS = SORT_BLOCK / 32;
 // 14 keys per thread (3584-key tiles) and four resident blocks per SM
 // measured fastest among 8-16 keys and 3-6 blocks on 16.6M ray keys; up to
 // SORT_MID_N keys, where larger tiles leave SMs idle and a pass is one tile's
-// latency, 7 (uniform / skewed 32-bit keys, 14 against 7: 100,000 keys 55 / 47
-// against 47 / 46 us, 250,000 56 / 54 against 55 / 47, 1M 76 / 65 against 84 / 73)
+// latency, 7 (uniform / skewed 32-bit keys, 14 against 7, measured before the passes'
+// launches overlapped: 100,000 keys 55 / 47 against 47 / 46 us, 250,000 56 / 54 against
+// 55 / 47, 1M 76 / 65 against 84 / 73; with them 35 / 33, 41 / 37 and, at 14, 65 / 55)
 constexpr int SORT_ITEMS = 14;
 constexpr int SORT_ITEMS_MID = 7;
 constexpr uint64_t SORT_MID_N = 450000;
@@ -588,7 +590,7 @@ __global__ void __launch_bounds__(SORT_BLOCK, WIDE ? WIDE_MIN_BLOCKS : SORT_MIN_
 
 // ------------------------------------------------------------ small sorts
 //
-// Up to 65,536 keys in one launch: a cluster of up to sixteen blocks of 1024
+// Up to 65,536 32-bit keys in one launch: a cluster of up to sixteen blocks of 1024
 // threads holds all (key, id) pairs in its shared memory.  Per digit pass
 // every thread takes its items into registers and ranks them within its warp
 // (rank_items), the block orders them by digit in shared memory while the
@@ -597,8 +599,8 @@ __global__ void __launch_bounds__(SORT_BLOCK, WIDE ? WIDE_MIN_BLOCKS : SORT_MIN_
 // one by one there instead took 1.2 cycles each, more than the rest of a pass).
 // The last pass's ids leave in whole lines.  Two cluster barriers a pass
 // replace the launches, the look-back and the round trips through L2 of the
-// general path, whose six launches cost the same 45 us or so at any size below
-// 200,000 keys.
+// general path, whose launches take 27 us for 32-bit keys at any size below.
+// 64-bit keys sort here if they fit one block.
 constexpr int SMALL_BLOCK = 1024;
 constexpr int SMALL_WARPS = SMALL_BLOCK / 32;
 constexpr int SMALL_ITEMS = 4;  // keys per thread (8 on half as many blocks: 47 against 35 us for 65,536 uniform keys)
@@ -669,7 +671,7 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
     constexpr bool PAIRS = sizeof(K) == 4;
     constexpr int QUARTER = SMALL_WARPS / 4;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t rank_in = cluster_rank(), blocks = cluster_size();
+    const uint32_t rank_in = PAIRS ? cluster_rank() : 0u, blocks = PAIRS ? cluster_size() : 1u;
     const uint32_t first = rank_in * SMALL_CAP;  // this block's positions
     const uint32_t tile_n = n > first ? min(n - first, SMALL_CAP) : 0u;
     const uint32_t wfirst = warp * (SMALL_ITEMS * 32) + lane;
@@ -791,8 +793,8 @@ cudaLaunchConfig_t small_config(unsigned blocks, cudaStream_t s, cudaLaunchAttri
 }
 
 // Blocks that a cluster of k_sort_small may have on device dev: 16 where the
-// device can place such a cluster, else the 8 that every device can (looked up,
-// with the kernel's shared-memory opt-in, once per device).
+// device can place such a cluster, else the 8 that every device can; a block alone
+// for 64-bit keys (looked up, with the kernel's shared-memory opt-in, once per device).
 template <typename K>
 cudaError_t small_blocks(int dev, unsigned *blocks) {
     static std::atomic<unsigned> known[64];
@@ -802,8 +804,8 @@ cudaError_t small_blocks(int dev, unsigned *blocks) {
     const auto kernel = k_sort_small<K>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared<K>));
     if (e != cudaSuccess) return e;
-    *blocks = 8;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    *blocks = sizeof(K) == 8 ? 1 : 8;
+    if (sizeof(K) == 4 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = small_config<K>(SMALL_CLUSTER, nullptr, attr);
         int clusters = 0;
@@ -817,13 +819,15 @@ cudaError_t small_blocks(int dev, unsigned *blocks) {
 template <typename K>
 cudaError_t run_sort(cudaStream_t s, const K *keys, uint32_t key_bits, uint64_t n, uint32_t *perm,
                      unsigned char *scratch, uint32_t *err, const SortOptions &opt) {
-    // One launch where the keys fit a cluster (measured against the general path,
-    // uniform / skewed 32-bit keys: 4,096 keys 24 / 19 against 49 / 47 us, 65,536
-    // keys 35 / 28 against 55 / 46; 64-bit keys 47 / 39 against 90 / 84 and 82 / 62
-    // against 100 / 84).  The withheld-tile test hook is about the general path's tiles.
+    // One launch where 32-bit keys fit a cluster or 64-bit keys a block (measured
+    // against the general path, uniform / skewed keys: 4,096 32-bit keys 17 / 13 against
+    // 29 / 27 us, 16,384 26 / 21 against 31 / 28, 65,536 32 / 26 against 33 / 31; 4,096
+    // 64-bit keys 35 / 26 against 48 / 46, but in a cluster 8,192 55 / 44 against 50 / 44
+    // and 65,536 82 / 62 against 61 / 55: eight exchanges cost more than eight
+    // launches that overlap).  The withheld-tile test hook is about the general path's tiles.
     int dev = 0;
     cudaGetDevice(&dev);
-    if (n <= SMALL_CLUSTER * SMALL_CAP && opt.withhold_tile == SortOptions().withhold_tile) {
+    if (n <= (sizeof(K) == 4 ? SMALL_CLUSTER * SMALL_CAP : SMALL_CAP) && opt.withhold_tile == SortOptions().withhold_tile) {
         unsigned most = 0, blocks = 1;
         const cudaError_t e = small_blocks<K>(dev, &most);
         if (e != cudaSuccess) return e;
