@@ -142,12 +142,14 @@ hcc_status hcc_reserve(hcc_ctx *ctx, uint64_t max_n, uint32_t max_key_bits);
  * How the context's traces schedule rays on warps.  PER_RAY: one thread per
  * ray slot for the whole traversal (the plain tracer).  REFILL: persistent
  * warps take ray slots from a counter in increasing order, and after each
- * traversal round the lanes whose ray has finished take new slots once 12
- * lanes of the warp are idle (24 when the rays are fetched through a sorted
- * permutation) (Aila & Laine 2009, "replacing terminated rays").  AUTO (the
+ * traversal round the lanes whose ray has finished take new slots once 8
+ * lanes of the warp are idle (over a layout's own nodes 12, or 24 when the rays
+ * are fetched through a sorted permutation) (Aila & Laine 2009, "replacing
+ * terminated rays").  AUTO (the
  * default): REFILL for closest-hit traces, PER_RAY for any-hit traces
  * (measured faster for each on GB300), and four threads per ray for
- * single wavefronts of at most 80,000 rays, which do not fill the GPU.  Results do not depend
+ * single wavefronts of at most 70,000 rays (any hit: 50,000), which do not
+ * fill the GPU.  Results do not depend
  * on the schedule, except which hit an any-hit query reports.
  */
 typedef enum hcc_trace_schedule {
@@ -379,8 +381,8 @@ hcc_status hcc_key_stats(hcc_ctx *ctx, const void *keys, uint32_t key_bits, cons
  * orders ray indices).  perm[j] = id of the j-th ray in sorted order.
  * keys: n uint32_t (key_bits <= 32) or uint64_t (key_bits > 32), device,
  * not modified.  perm: n uint32_t, device, must not overlap keys.
- * LSD radix sort, 8-bit digits: up to 65,536 keys in one launch, above that
- * one launch per digit, where digits that are equal for every key are
+ * LSD radix sort, 8-bit digits: up to 65,536 keys of at most 32 bits (4,096 of
+ * more) in one launch, above that one launch per digit, where digits that are equal for every key are
  * skipped, which leaves the result unchanged.  Scratch comes from the
  * context (see hcc_reserve).  n <= HCC_MAX_SORT_N.
  * Errors: INVALID_ARG, OOM, CUDA; TIMEOUT at hcc_sync if a bounded

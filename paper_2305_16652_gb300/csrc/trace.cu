@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(TRACE_BLOCK, LAYOUT == COMPACT ? 9 : 1) k_trac
 // rays: 563 against 321 us), so launch_layout keeps it to small wavefronts.
 // (Prefetching the met children's nodes: no change at 4,096 rays, 4 % slower at 65,536.)
 constexpr int QUAD_SLACK = 8;  // lanes that may still descend when the triangles are tested (0: 5 % slower, 16: 1 %)
-constexpr uint64_t QUAD_MAX_N = 80000;
+constexpr uint64_t QUAD_MAX_N = 70000, QUAD_MAX_N_ANY = 50000;
 constexpr uint32_t QUAD_MAX_LEVEL = 60;
 constexpr uint32_t QUAD_NONE = 0xFFFFFFFFu;
 
@@ -1185,19 +1185,22 @@ cudaError_t launch_pool_shaped(cudaStream_t s, const TraceArgs &a) {
 template <bool ANY, bool CNT, bool MULTI>
 cudaError_t launch_layout(cudaStream_t s, const TraceArgs &a, bool pool) {
     // Compact nodes wherever they exist and their deepest stack fits the trace's.
-    // They replaced each layout's own nodes by measurement (whole call, own against
-    // compact): 16.6M rays in HCC order over exact nodes 4.75 -> 3.95 ms, 0.96M
-    // 420 -> 323 us, 2.1M unsorted over wide nodes 614 -> 438 us, 2M in TwoPoint
-    // order over quantised nodes 745 -> 557 us, 4.1M shadow rays 640 -> 599 us.
+    // They replaced each layout's own nodes by measurement (the trace alone, exact nodes
+    // against compact: the room's 16.6M rays unsorted 4.79 -> 3.00 ms, in HCC order
+    // 3.97 -> 2.92, 33.2M shadow rays 3.82 -> 3.18 and 2.90 -> 2.49).  Rays so alike
+    // that the binary nodes stay in L1 gain least, as a step over four children is
+    // bound by its arithmetic: 16.6M rays off one patch of floor 3.76 -> 3.25 ms
+    // unsorted, but 3.01 -> 3.11 in HCC order and 2.63 -> 3.00 by origin and direction.
     if constexpr (!CNT) {
         const int depth = pool && !ANY ? a.stack : STACK;
         if (a.cstack <= (uint32_t)depth) {
             if constexpr (!MULTI) {
                 // Four lanes per ray where the rays do not fill the GPU (whole call, one
-                // lane against four: 4,096 rays 84 / 73 us, 20,000 84 / 67, 65,536 97 / 83,
-                // 40,000 unsorted 56 / 45, 30,000 shadow rays 79 / 71; 100,000 113 / 115,
-                // unsorted 68 / 77); a walk's levels are at most its stack entries.
-                if (a.quads && a.n <= QUAD_MAX_N && a.cstack <= QUAD_MAX_LEVEL) {
+                // lane against four: sorted 4,096 rays 76 / 55 us, 20,000 83 / 67, 65,536 96 /
+                // 86, 80,000 106 / 100; unsorted 40,000 60 / 45, 65,536 65 / 66, 80,000 69 /
+                // 71; shadow rays 40,000 51 / 48, 65,536 52 / 53, 80,000 60 / 65); a walk's
+                // levels are at most its stack entries.
+                if (a.quads && a.n <= (ANY ? QUAD_MAX_N_ANY : QUAD_MAX_N) && a.cstack <= QUAD_MAX_LEVEL) {
                     return launch_early(k_trace_quad<ANY>, (unsigned)((a.n + TRACE_BLOCK / 4 - 1) / (TRACE_BLOCK / 4)),
                                         TRACE_BLOCK, 0, s, a);
                 }
