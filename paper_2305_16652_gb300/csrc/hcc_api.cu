@@ -621,7 +621,7 @@ static uint32_t collapse_wide(const hcc_bvh_desc *d, std::vector<uint32_t> &word
 // suit the grid: not finite, a scene of extreme size, or boxes so small against
 // the scene that rounding them outward multiplies their summed surface, and with
 // it the expected node visits, by more than COMPACT_AREA (the compact walk is
-// 1.25 to 1.4 times as fast as the others' at the same visits).
+// 1.2 to 1.6 times as fast as the others' at the same visits, on rays of a whole room).
 struct CompactNodes {
     bool usable = false;
     std::vector<uint32_t> words;

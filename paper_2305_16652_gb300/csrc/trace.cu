@@ -42,13 +42,14 @@ constexpr uint32_t REFILL_MIN = 12;
 constexpr uint32_t REFILL_MIN_SORTED = 24;
 // ... and over compact nodes in either order: there a round is run by the whole
 // warp and costs little, so lanes need not wait as long (room's 16.6M rays in HCC
-// order, whole bounce: 3.97 ms at 8, 4.00 at 4 and 12, 4.20 at 24)
+// order, whole bounce: 3.74 ms at 8, 3.75 at 6, 3.73 at 10; with a heavier step 4.20
+// against 3.97 at 24)
 constexpr uint32_t REFILL_MIN_COMPACT = 8;
 // resident threads per SM the persistent kernel is built for; the register cap
 // follows from threads x registers <= 64K: exact and quantised binary nodes
 // (48 registers at 128-thread blocks), wide nodes or a batch of scenes (56), and
 // compact nodes (64; at 56 or 48 registers the loop spills and more warps share
-// the L1: 4.06 against 3.97 ms for the bounce above at 56, 72 registers 4.11)
+// the L1: 3.77 against 3.67 ms for the bounce above at 56; 72 registers 4.11 against 3.97)
 constexpr int pool_threads(int layout, bool multi) { return layout == 3 ? 1024 : layout == 2 || multi ? 1152 : 1280; }
 
 __device__ __forceinline__ float byte_to_float(uint32_t w, uint32_t sel) {
@@ -428,9 +429,10 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
 // nodes, seven 16-byte loads, 85 %) and waited for loads in 7.6 of 16 cycles per
 // instruction.  A compact node is read with two 32-byte loads for four children, so a
 // ray needs 16 visits and 33 loads where the binary nodes take 36 and 72, and the room's
-// nodes shrink from 32 to 13 MB.  What bounds the walk now (ncu, 0.96M rays): the
-// ALU pipe 71 %, issue 61 %, L1 data pipe 58 % busy, waits for loads 4.3 of 11.5
-// cycles per instruction; 154M warp instructions against 212M.
+// nodes shrink from 32 to 13 MB.  What bounds the walk now (ncu, 1.0M rays in
+// HCC order): the ALU pipe 63 %, issue 62 %, L1 data pipe 61 % busy at 21 lanes an
+// instruction, waits for loads 4.4 of 12.3 cycles per instruction; for 16.6M rays
+// 2.45 billion warp instructions against 3.41.
 
 // Traversal state over compact 4-ary nodes.  The slab test works in the
 // scene's grid: per axis tau = b * inv + c with b a decoded bound, inv the
@@ -638,7 +640,9 @@ __device__ __forceinline__ void compact_child(const CompactState &s, uint32_t wx
 // Entry distance of a child for the order of a step: its own if the ray meets it,
 // beyond any cap if it does not, by two multiply-adds where a compare and a
 // select would take the ALU pipe.  (A box missed by less than 1e-37 of the scene
-// may count as met, which costs a visit.)
+// may count as met, which costs a visit.)  With the best hit capping the pushes
+// alone, 12 of the step's ALU instructions less: 16.6M rays in HCC order, whole
+// bounce, 3.87 -> 3.77 ms, 2.1M unsorted 427 -> 414 us.
 constexpr float CAP_MAX = 8.0f;  // no box of the scene is met beyond 1
 __device__ __forceinline__ float met_distance(float tn, float tf) {
     return __fmaf_rn(__saturatef(__fsub_rn(tn, tf)), 1e38f, tn);
@@ -729,7 +733,7 @@ __device__ __forceinline__ float4 ldg_first(const float4 *p) {
 // step on branching, and pops alone in loops at 10 % of its lanes.  (The plain
 // rules for any hit, as for the other layouts: 592 us for 4.1M shadow rays and
 // their order against 596 with a slack of 4 lanes.)
-constexpr int COMPACT_SLACK = 6;    // 3: 1.5 % slower in HCC order, 5 % unsorted; 10: equal
+constexpr int COMPACT_SLACK = 6;    // 4: equal in HCC order, 1.8 % slower unsorted; 8: 0.3 % slower, 0.8 % faster
 constexpr int COMPACT_TRI_MIN = 6;  // 4 and 8 within 0.5 %
 template <bool ANY, bool FAR_C>
 __device__ __forceinline__ void ray_round(CompactState &s, const uint2 *stack, uint32_t stack_base,
