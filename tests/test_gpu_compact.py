@@ -100,3 +100,30 @@ def test_scene_that_does_not_suit_the_grid(ctx, layout):
     org[:, 3] = 0.0
     ref = _check(ctx, tris, org, dir_, layout)
     assert (ref["prim"] >= 0).any()
+
+
+@pytest.mark.parametrize("n", [2000, 100_000])
+def test_rays_in_the_planes_of_walls(ctx, n):
+    """Rays that run exactly in the plane of a room's wall, a face of the boxes above it, meet the
+    walls at its ends as the definition says (a slab test that takes 0 times the reciprocal of a
+    zero direction for an exit at t = 0 drops them)."""
+    box = np.array([[x, y, z] for x in (0, 10) for y in (0, 3) for z in (0, 8)], np.float32)
+    quads = [(0, 1, 3, 2), (4, 5, 7, 6), (0, 1, 5, 4), (2, 3, 7, 6), (0, 2, 6, 4), (1, 3, 7, 5)]
+    walls = [box[[a, b, c]].reshape(9) for q in quads for a, b, c in (q[:3], (q[0], q[2], q[3]))]
+    tris = np.ascontiguousarray(np.concatenate([np.array(walls, np.float32), gen.random_tris(9, 100, mu=-1.5)]))
+    rng = np.random.default_rng(17)
+    axis, side = rng.integers(0, 3, 2000), rng.integers(0, 2, 2000)
+    o, d = rng.random((2000, 3)) * [8, 2, 6] + [1, 0.5, 1], rng.normal(size=(2000, 3))
+    rows = np.arange(2000)
+    o[rows, axis] = np.array([10.0, 3.0, 8.0])[axis] * side
+    d[rows, axis] = 0.0
+    org = np.concatenate([o, np.full((2000, 1), 1e-4)], 1).astype(np.float32)
+    dir_ = np.concatenate([d, np.full((2000, 1), np.inf)], 1).astype(np.float32)
+    ref = oracle.trace_brute(tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 500
+    h = hcc.hcc_bvh_upload(ctx, gen.build_bvh(tris), layout="exact")
+    try:
+        got = _trace(ctx, h, np.tile(org, (n // 2000, 1)), np.tile(dir_, (n // 2000, 1)))
+        assert np.array_equal(got.view(np.int32), np.tile(ref, n // 2000).view(np.int32))
+    finally:
+        hcc.hcc_bvh_destroy(h)
