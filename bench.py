@@ -46,7 +46,9 @@ SMS, LANES_PER_SM = 152, 128
 # Moller-Trumbore sequence (~45 ops incl. the reciprocal).  A 4-ary node
 # visit (wide layout) runs four directed slab tests (6 fma, 5 min/max/mul,
 # 4 to mark and clamp the met child = 15 each), selects its near/far rows
-# (9), sorts the four entries (5 exchanges of 5 ops) and pushes (~12).
+# (9), sorts the four entries (5 exchanges of 5 ops) and pushes (~12).  The
+# counts are visits of the layout's own nodes (the counting diagnostic walks
+# them), the same work whichever nodes the timed trace walks.
 OPS_PER_NODE = {"exact": 2 * 26 + 10, "quantised": 36 + 6 + 2 * 26 + 10, "wide": 4 * 15 + 9 + 25 + 12}
 OPS_PER_TRI = 45
 # HBM bytes each stage must move per ray (32-bit keys; see the design notes)
