@@ -516,6 +516,16 @@ __device__ __forceinline__ float grid_inv(float d) {
     return r;
 }
 
+// Reciprocal of a grid-space direction in tau, limited so that its products with
+// grid coordinates (below GRID_REACH) stay finite: for a component that grid_inv replaced, the
+// scale of a ray that leaves the scene soon would take them to infinity, which
+// is neither before nor behind the ray.  At the limit the smallest gap between two bounds
+// is still 1e31 in tau, as wide as an axis that the ray does not move along has to be.
+constexpr float TAU_INV_MAX = 1e36f;
+__device__ __forceinline__ float scaled_inv(float inv, float scale) {
+    return fminf(fmaxf(__fmul_rn(inv, scale), -TAU_INV_MAX), TAU_INV_MAX);
+}
+
 // A lane without a ray.
 __device__ __forceinline__ void ray_none(CompactState &s, uint32_t stack_base) {
     s.node = s.leaf = REF_NONE;
@@ -546,7 +556,7 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
         meets = enter_grid(o4, d4, g, p, from);
         start = 0.0f;
     }
-    // c, and the far side of the scene, in t from `from`
+    // the far side of the scene, in t from `from`
     const float cx = __fmaf_rn(-p.x, ix, -start), cy = __fmaf_rn(-p.y, iy, -start), cz = __fmaf_rn(-p.z, iz, -start);
     const float leave = fmin3(__fmaf_rn(ix < 0.0f ? 2.0f : 8.0f, ix, cx), __fmaf_rn(iy < 0.0f ? 2.0f : 8.0f, iy, cy),
                               __fmaf_rn(iz < 0.0f ? 2.0f : 8.0f, iz, cz));
@@ -555,10 +565,13 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     const uint32_t e = __float_as_uint(fmaxf(leave, 2e-38f)) >> 23;
     const float scale = __uint_as_float((252u - (e < 251u ? e : 251u)) << 23);
     meets = meets && leave > 0.0f && tmax > 0.0f;
-    s.ixy = make_float2(__fmul_rn(ix, scale), __fmul_rn(iy, scale));
-    s.iz = __fmul_rn(iz, scale);
-    s.cxy = make_float2(__fmul_rn(cx, scale), __fmul_rn(cy, scale));
-    s.cz = __fmul_rn(cz, scale);
+    // c from the limited reciprocal: the same bits as c * scale where the limit does not bind
+    const float jx = scaled_inv(ix, scale), jy = scaled_inv(iy, scale), jz = scaled_inv(iz, scale);
+    const float from_tau = __fmul_rn(-start, scale);
+    s.ixy = make_float2(jx, jy);
+    s.iz = jz;
+    s.cxy = make_float2(__fmaf_rn(-p.x, jx, from_tau), __fmaf_rn(-p.y, jy, from_tau));
+    s.cz = __fmaf_rn(-p.z, jz, from_tau);
     s.sx = ix < 0.0f ? 0x4325u : 0x4105u;
     s.sy = iy < 0.0f ? 0x4325u : 0x4105u;
     s.sz = iz < 0.0f ? 0x4325u : 0x4105u;

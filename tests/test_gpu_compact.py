@@ -21,15 +21,20 @@ def ctx():
 
 
 def _check(ctx, tris, org, dir_, layout="exact"):
+    """Closest and any hits against brute force, by each walk: four lanes per ray (auto, for this
+    many rays), one thread per ray, and warps that take new rays."""
     bvh = gen.build_bvh(tris)
     h = hcc.hcc_bvh_upload(ctx, bvh, layout=layout)
     try:
         ref = oracle.trace_brute(tris, org, dir_)
-        compare_hits(_trace(ctx, h, org, dir_), ref)
-        occl = _trace(ctx, h, org, dir_, any_hit=True)["prim"] >= 0
-        assert np.array_equal(occl, ref["prim"] >= 0)
+        for schedule in ("auto", "per_ray", "refill"):
+            hcc.hcc_set_trace_schedule(ctx, schedule)
+            compare_hits(_trace(ctx, h, org, dir_), ref)
+            occl = _trace(ctx, h, org, dir_, any_hit=True)["prim"] >= 0
+            assert np.array_equal(occl, ref["prim"] >= 0), schedule
         return ref
     finally:
+        hcc.hcc_set_trace_schedule(ctx, "auto")
         hcc.hcc_bvh_destroy(h)
 
 
@@ -127,3 +132,85 @@ def test_rays_in_the_planes_of_walls(ctx, n):
         assert np.array_equal(got.view(np.int32), np.tile(ref, n // 2000).view(np.int32))
     finally:
         hcc.hcc_bvh_destroy(h)
+
+
+def _axis_parallel(rng, n, zeros, o):
+    """Rays from o in directions with `zeros` zero components, of either sign, and either sign of zero."""
+    d = rng.normal(size=(n, 3))
+    order = np.argsort(rng.random((n, 3)), axis=1)
+    for k in range(zeros):
+        d[np.arange(n), order[:, k]] = np.where(rng.random(n) < 0.5, 0.0, -0.0)
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    org = np.concatenate([o, np.zeros((n, 1))], 1).astype(np.float32)
+    return org, np.concatenate([d, np.full((n, 1), np.inf)], 1).astype(np.float32)
+
+
+@pytest.mark.parametrize("zeros", [1, 2])
+@pytest.mark.parametrize("scale", [1e-4 * 2.0**k for k in range(11)])
+def test_zero_components_in_small_scenes(ctx, scale, zeros):
+    """The far side of the scene lies 1e-4 to 0.1 ahead: the ray's scale is large, and the
+    reciprocal of a zero component must not go to infinity with it."""
+    tris = (gen.random_tris(37, 400, mu=-1.5) * np.float32(scale)).astype(np.float32)
+    rng = np.random.default_rng(zeros)
+    org, dir_ = _axis_parallel(rng, 2000, zeros, rng.random((2000, 3)) * scale)
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 300
+
+
+@pytest.mark.parametrize("zeros", [1, 2])
+@pytest.mark.parametrize("length", [1e-6, 1e-3, 1e3, 2e3, 4e3, 1e4, 1e5, 1e6])
+def test_zero_components_and_direction_lengths(ctx, length, zeros):
+    tris = (gen.random_tris(41, 400, mu=-1.5) * np.float32(10)).astype(np.float32)
+    rng = np.random.default_rng(zeros)
+    org, dir_ = _axis_parallel(rng, 2000, zeros, rng.random((2000, 3)) * 10)
+    dir_[:, :3] *= np.float32(length)
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 300
+
+
+@pytest.mark.parametrize("zeros", [1, 2])
+@pytest.mark.parametrize("ahead", [0.0005, 0.001, 0.002, 0.004, 0.006, 0.01])
+def test_zero_components_just_before_an_outer_wall(ctx, ahead, zeros):
+    """A wall at the edge of a scene of one unit, a little ahead of the rays."""
+    rng = np.random.default_rng(zeros)
+    wall = np.array([[1, -1, -1, 1, 2, -1, 1, 2, 2], [1, -1, -1, 1, 2, 2, 1, -1, 2]], np.float32)
+    tris = np.ascontiguousarray(np.concatenate([np.clip(gen.random_tris(43, 400, mu=-1.5), 0, 0.9), wall])).astype(np.float32)
+    o = rng.random((2000, 3))
+    o[:, 0] = 1 - ahead
+    org, dir_ = _axis_parallel(rng, 2000, zeros, o)
+    dir_[:, 0] = np.abs(dir_[:, 0])
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 400).sum() > 300
+
+
+def test_zero_components_in_a_batch_and_a_server(ctx):
+    scales = (0.002, 0.004, 1.0)
+    rng = np.random.default_rng(47)
+    tris = [(gen.random_tris(51 + k, 400, mu=-1.5) * np.float32(s)).astype(np.float32) for k, s in enumerate(scales)]
+    rays = [_axis_parallel(rng, 1000, 1, rng.random((1000, 3)) * s) for s in scales]
+    refs = [oracle.trace_brute(t, *r) for t, r in zip(tris, rays)]
+    bvhs = [hcc.hcc_bvh_upload(ctx, gen.build_bvh(t), layout="exact") for t in tris]
+    cuts = [hcc.hcc_select_cut(ctx, b, 16, 0.125) for b in bvhs]
+    batch = hcc.hcc_batch_create(ctx, bvhs, cuts, [0, 1000, 2000, 3000])
+    server = hcc.hcc_server_create(0, bvhs, cuts, slots=2, method="hcc", key_bits=16)
+    try:
+        o, d = (torch.from_numpy(np.concatenate([r[k] for r in rays])).to("cuda:0") for k in (0, 1))
+        hits = torch.zeros((3000, 4), dtype=torch.int32, device="cuda:0")
+        hcc.hcc_batch_run(ctx, batch, "hcc", o, d, 16, hits)
+        hcc.hcc_sync(ctx)
+        compare_hits(hcc.hits_to_numpy(hits), np.concatenate(refs))
+        for k, (r, ref) in enumerate(zip(rays, refs)):
+            for any_hit in (False, True):
+                got = np.zeros(1000, oracle.HIT_DTYPE)
+                hcc.hcc_server_wait(server, hcc.hcc_server_submit(server, k, *r, got, any_hit=any_hit))
+                if any_hit:
+                    assert np.array_equal(got["prim"] >= 0, ref["prim"] >= 0)
+                else:
+                    compare_hits(got, ref)
+    finally:
+        hcc.hcc_server_destroy(server)
+        hcc.hcc_batch_destroy(batch)
+        for c in cuts:
+            hcc.hcc_cut_destroy(c)
+        for b in bvhs:
+            hcc.hcc_bvh_destroy(b)
