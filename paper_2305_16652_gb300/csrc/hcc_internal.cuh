@@ -49,9 +49,12 @@ constexpr uint32_t REF_TRI_MASK = 0x1FFFFFFFu;
 constexpr float GRID_ORIGIN = 2.0009765625f;     // 2 + 2^-10
 constexpr float GRID_SPAN = 5.9921875f;          // 6 - 2^-7: M(hi) stays below 8 - 2^-8
 constexpr float GRID_MARGIN = 3.147125244e-05f;  // 2^-15 + 2^-20, half the grid's smallest step
-// A ray whose origin lies further than this from the grid's zero is traced
-// from the point where it enters the scene: within it, the rounding of the
-// ray's grid coordinates and of its slab distances stays below GRID_MARGIN.
+// A ray whose origin lies further than this from the grid's zero, or its start (tmin)
+// further behind its origin on an axis, is traced from the point where it enters the
+// scene.  Within these limits the rounding of the ray's grid coordinates and of its slab
+// distances stays below GRID_MARGIN.  In 2^-24 grid units: origin less grid.lo 32 and its
+// fma 16, the reciprocal 3 for each of at most 40 units from the origin, c and tau (each
+// at most 72 units, a start further ahead being beyond the scene) 64 each: 296, or 1.8e-5.
 constexpr float GRID_REACH = 32.0f;
 
 struct Grid {

@@ -440,7 +440,7 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
 // bound.  Its rounding, and that of the ray's grid coordinates, is below the
 // margin by which the stored bounds were widened, so no factor on the far
 // distance is needed.  tau is the ray's parameter t measured from `from` (tmin, or
-// the entry into the scene for an origin far outside it) and scaled by a power
+// the entry into the scene for an origin or a tmin far outside it) and scaled by a power
 // of two that brings the scene's far side below 1: a saturating fma then
 // clamps the entry distance to the ray's start.
 struct CompactState {
@@ -476,10 +476,11 @@ __device__ __forceinline__ float grid_bound(uint32_t w, uint32_t sel) {
     return __uint_as_float(__byte_perm(w, 0x40u, sel));
 }
 
-// A ray whose origin is more than GRID_REACH from the grid's zero: measures t
+// A ray whose origin is more than GRID_REACH from the grid's zero, or whose
+// interval starts further than that from its origin (tmin far below zero): measures t
 // from the point where it enters the scene's neighbourhood (one unit around the
 // grid's box), computed in double, so that the grid coordinates of the slab test
-// stay small.  Returns false if it never comes near.
+// and the distances it takes from them stay small.  Returns false if it never comes near.
 __device__ __noinline__ bool enter_grid(const float4 o4, const float4 d4, const Grid &g, float3 &p, float &from) {
     const float o[3] = {o4.x, o4.y, o4.z}, d[3] = {d4.x, d4.y, d4.z};
     double op[3], dp[3], tin = (double)o4.w, tout = (double)d4.w;
@@ -547,10 +548,12 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     float3 p = make_float3(__fmaf_rn(__fsub_rn(o4.x, g.lo[0]), g.scale[0], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.y, g.lo[1]), g.scale[1], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.z, g.lo[2]), g.scale[2], GRID_ORIGIN));
-    const float ix = grid_inv(__fmul_rn(d4.x, g.scale[0])), iy = grid_inv(__fmul_rn(d4.y, g.scale[1])),
-                iz = grid_inv(__fmul_rn(d4.z, g.scale[2]));
+    const float gx = __fmul_rn(d4.x, g.scale[0]), gy = __fmul_rn(d4.y, g.scale[1]), gz = __fmul_rn(d4.z, g.scale[2]);
+    const float ix = grid_inv(gx), iy = grid_inv(gy), iz = grid_inv(gz);
     float from = o4.w, start = o4.w;  // start: `from` as seen from p
-    const bool far = fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)) > GRID_REACH;
+    // (a tmin that far above zero is beyond the scene, and the ray a miss below)
+    const bool far = fmaxf(fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)),
+                           __fmul_rn(-start, fmax3(fabsf(gx), fabsf(gy), fabsf(gz)))) > GRID_REACH;
     bool meets = true;
     if (far) {
         meets = enter_grid(o4, d4, g, p, from);

@@ -214,3 +214,17 @@ def test_zero_components_in_a_batch_and_a_server(ctx):
             hcc.hcc_cut_destroy(c)
         for b in bvhs:
             hcc.hcc_bvh_destroy(b)
+
+
+@pytest.mark.parametrize("size", [1.0, 10.0])
+@pytest.mark.parametrize("tmin", [-1e2, -3e2, -1e3, -1e4, -1e5, -1e6, -1e8, -1e30, -np.inf])
+def test_intervals_that_start_far_behind_the_origin(ctx, tmin, size):
+    """Rays measured from a tmin far below zero meet what they meet from a nearer one."""
+    tris = (gen.random_tris(61, 2000, mu=-3.0) * np.float32(size)).astype(np.float32)
+    org, dir_ = _rays(67, 6000, tris)
+    org[:, 3] = tmin
+    dir_[::2, 3] = 0.0  # nothing ahead of the origin
+    dir_[1::3, 0] = 0.0
+    dir_[2::9, :2] = 0.0
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 300 and (ref["t"] < 0).sum() > 100
