@@ -161,6 +161,22 @@ typedef enum hcc_trace_schedule {
 hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule);
 
 /*
+ * Nodes that the context's traces walk, single wavefronts and batches.  AUTO
+ * (the default): the compact nodes where the BVH has them and its deepest stack
+ * fits, else its layout's (see hcc_bvh_layout).  LAYOUT: always its layout's,
+ * for programs whose rays are so alike that these stay in L1 (sorted rays off
+ * one patch of floor: exact nodes 3 to 14 % faster).  Results do not depend on
+ * it, except which hit an any-hit query reports.  Servers use AUTO.
+ * Errors: INVALID_ARG for another value.
+ */
+typedef enum hcc_trace_nodes {
+    HCC_TRACE_NODES_AUTO = 0,
+    HCC_TRACE_NODES_LAYOUT = 1
+} hcc_trace_nodes;
+
+hcc_status hcc_set_trace_nodes(hcc_ctx *ctx, hcc_trace_nodes nodes);
+
+/*
  * Shape of the context's closest-hit traces that use ray replacement
  * (REFILL, and AUTO for closest hit), single wavefronts and batches: threads
  * per block (64, 128 or 256) and traversal-stack entries per ray (32, 48 or
@@ -238,8 +254,9 @@ typedef enum hcc_bvh_layout {
  * boxes do not suit them: a scene wider than 1e9 or narrower than 1e-9 units, or
  * boxes so small against it that the grid would add a fifth to their surface.
  * Traces (single, batches, servers) walk the compact nodes where their deepest
- * stack fits the trace's; the layout's nodes are what they walk otherwise, what
- * hcc_trace_counts counts and what the prefix path code reads. */
+ * stack fits the trace's, unless hcc_set_trace_nodes says otherwise; else they
+ * walk the layout's nodes, which are also what hcc_trace_counts counts and what
+ * the prefix path code reads. */
 
 /* hcc_bvh_upload with a choice of node layout.  Every layout gives the same
  * hits (boxes only decide which triangles are tested, and every box holds

@@ -44,6 +44,7 @@ struct hcc_ctx {
     uint32_t *d_err = nullptr;                 // device error word, followed by ...
     hcc::TraceWork *d_work = nullptr;          // ... the trace's counters
     hcc_trace_schedule schedule = HCC_TRACE_AUTO;
+    hcc_trace_nodes nodes = HCC_TRACE_NODES_AUTO;
     float twopoint_fraction = 0.25f;            // TwoPoint length estimate / largest extent
     hcc::SortOptions sort_opt;                  // bounded-wait settings of this context's sorts
     uint32_t trace_block = 128, trace_stack = HCC_TRACE_STACK;  // shape of the closest-hit persistent trace
@@ -356,6 +357,11 @@ static TraceWork *trace_work(const hcc_ctx *ctx, int any_hit) {
     return refill ? ctx->d_work : nullptr;
 }
 
+// Stack entries for which a trace may walk compact nodes of depth `stack`: none where the context asks for the layout's.
+static uint32_t trace_cstack(const hcc_ctx *ctx, uint32_t stack) {
+    return ctx->nodes == HCC_TRACE_NODES_LAYOUT ? 0xFFFFFFFFu : stack;
+}
+
 // What the traces of one BVH share: the scene, the rays and the context's settings.
 static TraceArgs trace_args(const hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_rays *rays, int any_hit) {
     TraceArgs a;
@@ -365,7 +371,7 @@ static TraceArgs trace_args(const hcc_ctx *ctx, const hcc_bvh *bvh, const hcc_ra
     a.root_ref = bvh->root_ref;
     a.cnodes = bvh->d_compact;
     a.croot = bvh->compact_root;
-    a.cstack = bvh->compact_stack;
+    a.cstack = trace_cstack(ctx, bvh->compact_stack);
     a.grid = bvh->grid;
     a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
     a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
@@ -433,6 +439,14 @@ hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule) {
     if (schedule != HCC_TRACE_AUTO && schedule != HCC_TRACE_PER_RAY && schedule != HCC_TRACE_REFILL)
         return fail(ctx, HCC_ERR_INVALID_ARG, "unknown trace schedule");
     ctx->schedule = schedule;
+    return HCC_OK;
+}
+
+hcc_status hcc_set_trace_nodes(hcc_ctx *ctx, hcc_trace_nodes nodes) {
+    if (!ctx) return HCC_ERR_INVALID_ARG;
+    if (nodes != HCC_TRACE_NODES_AUTO && nodes != HCC_TRACE_NODES_LAYOUT)
+        return fail(ctx, HCC_ERR_INVALID_ARG, "unknown trace nodes");
+    ctx->nodes = nodes;
     return HCC_OK;
 }
 
@@ -1453,7 +1467,7 @@ hcc_status hcc_batch_run(hcc_ctx *ctx, const hcc_batch *b, hcc_method method, co
     DeviceGuard g(ctx->device);
     TraceArgs a;
     a.layout = b->layout;
-    a.cstack = b->compact_stack;
+    a.cstack = trace_cstack(ctx, b->compact_stack);
     a.org = reinterpret_cast<const float4 *>(rays->org_tmin);
     a.dir = reinterpret_cast<const float4 *>(rays->dir_tmax);
     a.rs = ray_rs(rays);
@@ -1684,6 +1698,7 @@ hcc_status hcc_run_host(hcc_ctx *ctx, hcc_method method, const hcc_bvh *bvh, con
     }
     for (hcc_ctx *l : ctx->lane) {  // the lanes follow the context's settings
         l->schedule = ctx->schedule;
+        l->nodes = ctx->nodes;
         l->trace_block = ctx->trace_block;
         l->trace_stack = ctx->trace_stack;
         l->twopoint_fraction = ctx->twopoint_fraction;

@@ -79,6 +79,7 @@ def load(path: str = LIB_PATH):
         "hcc_destroy": [P],
         "hcc_set_stream": [P, P],
         "hcc_set_trace_schedule": [P, i32],
+        "hcc_set_trace_nodes": [P, i32],
         "hcc_set_twopoint_distance": [P, ctypes.c_float],
         "hcc_set_sort_wait_limit": [P, u32],
         "hcc_set_trace_shape": [P, u32, u32],
@@ -253,6 +254,14 @@ TRACE_SCHEDULES = {"auto": 0, "per_ray": 1, "refill": 2}
 def hcc_set_trace_schedule(ctx, schedule="auto"):
     """Ray scheduling of the context's traces: auto, per_ray or refill."""
     _check(load().hcc_set_trace_schedule(ctx, TRACE_SCHEDULES.get(schedule, schedule)), ctx)
+
+
+TRACE_NODES = {"auto": 0, "layout": 1}
+
+
+def hcc_set_trace_nodes(ctx, nodes="auto"):
+    """Nodes that the context's traces walk: auto (compact where possible) or layout."""
+    _check(load().hcc_set_trace_nodes(ctx, TRACE_NODES.get(nodes, nodes)), ctx)
 
 
 def hcc_set_twopoint_distance(ctx, fraction: float = 0.25):

@@ -26,9 +26,11 @@ def _scenes():
     return ws
 
 
-@pytest.fixture(scope="module")
-def env():
+@pytest.fixture(scope="module", params=["auto", "layout"])
+def env(request):
+    """Traces over the compact nodes, and over the layouts' own."""
     ctx = hcc.hcc_create(0)
+    hcc.hcc_set_trace_nodes(ctx, request.param)
     ws = _scenes()
     layouts = {}
     for layout in ("exact", "quantised", "wide"):

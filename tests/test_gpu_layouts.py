@@ -21,9 +21,11 @@ DEV = "cuda:0"
 LAYOUTS = ("quantised", "exact", "wide")
 
 
-@pytest.fixture(scope="module")
-def ctx():
+@pytest.fixture(scope="module", params=["auto", "layout"])
+def ctx(request):
+    """Traces over the compact nodes, and over the layout's own."""
     c = hcc.hcc_create(0)
+    hcc.hcc_set_trace_nodes(c, request.param)
     yield c
     hcc.hcc_destroy(c)
 

@@ -425,6 +425,15 @@ def test_ray_stride_must_be_a_multiple_of_16(ctx, room):
 
 # ------------------------------------------------------------------- trace
 
+@pytest.fixture(params=["auto", "layout"])
+def nodes(request, ctx):
+    """Traces over the compact nodes, and over the layouts' own."""
+    hcc.hcc_set_trace_nodes(ctx, request.param)
+    yield request.param
+    hcc.hcc_set_trace_nodes(ctx, "auto")
+
+
+@pytest.mark.usefixtures("nodes")
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
 @pytest.mark.parametrize("which", ["tiny", "dense", "room"])
 def test_trace_closest_matches_oracle(ctx, which, layout, request):
@@ -435,6 +444,7 @@ def test_trace_closest_matches_oracle(ctx, which, layout, request):
     assert (g["prim"] >= 0).mean() > 0.2
 
 
+@pytest.mark.usefixtures("nodes")
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
 def test_trace_matches_brute_force_definition(ctx, dense, layout):
     g = gpu_trace(ctx, dense, dense.org, dense.dir, layout=layout)
@@ -442,6 +452,7 @@ def test_trace_matches_brute_force_definition(ctx, dense, layout):
     compare_hits(g, o)
 
 
+@pytest.mark.usefixtures("nodes")
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
 def test_trace_any_hit_shadow_rays(ctx, room, layout):
     sh = room.w.shadow
@@ -457,6 +468,7 @@ def test_trace_any_hit_shadow_rays(ctx, room, layout):
         assert ok and np.float32(t) == g["t"][i]
 
 
+@pytest.mark.usefixtures("nodes")
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
 def test_trace_special_rays(ctx, dense, layout):
     rng = np.random.default_rng(1)
@@ -477,6 +489,7 @@ def test_trace_special_rays(ctx, dense, layout):
     assert np.all(g["prim"][200:230] == -1)
 
 
+@pytest.mark.usefixtures("nodes")
 def test_trace_scatter_and_reorder_invariance(ctx, room):
     rng = np.random.default_rng(3)
     perm = rng.permutation(room.n).astype(np.uint32)
@@ -641,6 +654,7 @@ def test_trace_shape_stack_depth_is_honoured(ctx, tiny, layout):
         hcc.hcc_bvh_destroy(h)
 
 
+@pytest.mark.usefixtures("nodes")
 @pytest.mark.parametrize("which", ["tiny", "room"])
 def test_trace_schedules_give_the_same_records(ctx, which, request):
     """One thread per ray and the persistent trace with ray replacement return
@@ -673,6 +687,8 @@ def test_trace_schedules_give_the_same_records(ctx, which, request):
             assert c["warp_node_steps"] <= c["node_visits"] <= 32 * c["warp_node_steps"]
         with pytest.raises(hcc.HccError):
             hcc.hcc_set_trace_schedule(ctx, 7)
+        with pytest.raises(hcc.HccError):
+            hcc.hcc_set_trace_nodes(ctx, 2)
     finally:
         hcc.hcc_set_trace_schedule(ctx, "auto")
         hcc.hcc_cut_destroy(cut)
