@@ -228,3 +228,60 @@ def test_intervals_that_start_far_behind_the_origin(ctx, tmin, size):
     dir_[2::9, :2] = 0.0
     ref = _check(ctx, tris, org, dir_)
     assert (ref["prim"] >= 0).sum() > 300 and (ref["t"] < 0).sum() > 100
+
+
+def _trace_us(ctx, h, org, dir_, nodes, any_hit):
+    hits = torch.zeros((org.shape[0], 4), dtype=torch.int32, device="cuda:0")
+    hcc.hcc_set_trace_nodes(ctx, nodes)
+    times = []
+    for _ in range(7):
+        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        start.record()
+        for _ in range(5):
+            hcc.hcc_trace(ctx, h, org, dir_, hits, any_hit=any_hit)
+        end.record()
+        end.synchronize()
+        times.append(start.elapsed_time(end) * 200)
+    hcc.hcc_set_trace_nodes(ctx, "auto")
+    hcc.hcc_sync(ctx)
+    return float(np.median(times)), hits.cpu().numpy()
+
+
+def _detail(ground):
+    """An object of 0.3 units (a bumpy ball of 100,000 triangles) on a ground of the given size, and rays
+    at it from about 0.6 units away."""
+    rng = np.random.default_rng(71)
+    m = 224
+    a, b = np.meshgrid(np.linspace(0, 2 * np.pi, m + 1), np.linspace(0.02, np.pi - 0.02, m + 1), indexing="ij")
+    r = 0.15 * (1 + 0.004 * rng.normal(size=a.shape))
+    p = np.stack([r * np.cos(a) * np.sin(b), 0.15 + r * np.cos(b), r * np.sin(a) * np.sin(b)], -1)
+    q = [p[:-1, :-1], p[1:, :-1], p[1:, 1:], p[:-1, 1:]]
+    g = ground / 2
+    plane = [[-g, 0, -g, g, 0, -g, g, 0, g], [-g, 0, -g, g, 0, g, -g, 0, g]]
+    tris = np.concatenate([np.concatenate([q[0], q[i], q[i + 1]], -1).reshape(-1, 9) for i in (1, 2)] + [np.array(plane)])
+    o = rng.normal(size=(500_000, 3))
+    o *= 0.6 / np.linalg.norm(o, axis=1, keepdims=True)
+    o[:, 1] = 0.15 + np.abs(o[:, 1])
+    d = rng.normal(scale=0.07, size=o.shape) + [0, 0.15, 0] - o
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    pad = [np.full((o.shape[0], 1), x) for x in (1e-4, np.inf)]
+    return tris.astype(np.float32), *(np.concatenate([x, y], 1).astype(np.float32) for x, y in zip((o, d), pad))
+
+
+@pytest.mark.parametrize("ground", [1.0, 30.0, 100.0, 1000.0])
+def test_small_detail_in_large_scenes_costs_no_more_than_the_layouts_nodes(ctx, ground):
+    """The grid spans the scene, so its step grows with it; rays at an object that the step is coarse
+    for must not pay for it (exact nodes: 1.3 times slower on the smallest ground, as on rooms)."""
+    tris, org, dir_ = _detail(ground)
+    h = hcc.hcc_bvh_upload(ctx, gen.build_bvh(tris), layout="exact")
+    try:
+        o, d = torch.from_numpy(org).to("cuda:0"), torch.from_numpy(dir_).to("cuda:0")
+        for any_hit in (False, True):
+            (t_auto, hit), (t_layout, ref) = (_trace_us(ctx, h, o, d, x, any_hit) for x in ("auto", "layout"))
+            assert np.array_equal(hit[:, 0] >= 0, ref[:, 0] >= 0)
+            assert any_hit or (hit != ref).any(axis=1).sum() <= 5  # ties on an edge
+            assert t_auto < 1.15 * t_layout
+            if ground == 1.0:
+                assert t_auto < t_layout
+    finally:
+        hcc.hcc_bvh_destroy(h)
