@@ -94,6 +94,26 @@ __device__ __forceinline__ void slab(const Ray &r, const Box2 &b, float tcap, fl
     tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
 }
 
+// A ray with a zero direction component may lie in the plane of a box's face, where the
+// reciprocal that stands in for infinity gives an entry or exit at t = 0.  For
+// such rays a distance of zero is taken as beyond either end.  (The check costs
+// the walk of exact and quantised nodes 0.3 to 1.6 %; applied to every ray it cost
+// 5 to 30 %, as rays that start on a wall then test the wall.)
+__device__ __forceinline__ bool flat_ray(const Ray &r) {
+    return fmax3(fabsf(r.ixy.x), fabsf(r.ixy.y), fabsf(r.izz.x)) > 0.9e30f;  // safe_inv's stand-in is 1e30
+}
+__device__ __forceinline__ float flat_near(float t) { return t == 0.0f ? -__int_as_float(0x7F800000) : t; }
+__device__ __forceinline__ float flat_far(float t) { return t == 0.0f ? __int_as_float(0x7F800000) : t; }
+
+__device__ __forceinline__ void slab_flat(const Ray &r, const Box2 &b, float tcap, float &tn, float &tf) {
+    const float2 a = __fmul2_rn(__fadd2_rn(b.lxy, r.nxy), r.ixy);
+    const float2 c = __fmul2_rn(__fadd2_rn(b.hxy, r.nxy), r.ixy);
+    const float2 z = __fmul2_rn(__fadd2_rn(b.zz, r.nzz), r.izz);
+    tn = fmax3(flat_near(fminf(a.x, c.x)), flat_near(fminf(a.y, c.y)), fmaxf(flat_near(fminf(z.x, z.y)), r.tmin));
+    const float f = fmin3(flat_far(fmaxf(a.x, c.x)), flat_far(fmaxf(a.y, c.y)), flat_far(fmaxf(z.x, z.y)));
+    tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
+}
+
 // Moller-Trumbore; returns true with (t, u, v) if the ray's line meets the
 // triangle (the caller checks t against the ray's interval).  Same operation sequence as the definition: p = d x e2,
 // det = e1 . p, s = o - v0, u = (s . p) / det, q = s x e1, v = (d . q) / det,
@@ -220,6 +240,19 @@ struct RayState {
     bool overflow;
 };
 
+// o * inv rounded down and up, for wide nodes.  For a zero direction component they
+// are moved apart by 1e20 or four places, so that a ray in the plane of a
+// box's face lies within the box (as slab_flat does for binary nodes).
+__device__ __forceinline__ void scaled_origin(float o, float d, float inv, float &down, float &up) {
+    down = __fmul_rd(o, inv);
+    up = __fmul_ru(o, inv);
+    if (!(fabsf(d) > 1e-30f)) {
+        const float apart = fmaxf(fabsf(up) * 0x1p-22f, 1e20f);
+        down = __fsub_rd(down, apart);
+        up = __fadd_ru(up, apart);
+    }
+}
+
 __device__ __forceinline__ void ray_init(RayState &s, const float4 o4, const float4 d4, uint32_t root_ref) {
     s.r.nxy = make_float2(-o4.x, -o4.y);
     s.r.nzz = make_float2(-o4.z, -o4.z);
@@ -231,12 +264,9 @@ __device__ __forceinline__ void ray_init(RayState &s, const float4 o4, const flo
     const float ix = safe_inv(d4.x), iy = safe_inv(d4.y), iz = safe_inv(d4.z);
     s.r.ixy = make_float2(ix, iy);
     s.r.izz = make_float2(iz, iz);
-    s.r.lx = __fmul_rd(o4.x, ix);
-    s.r.ly = __fmul_rd(o4.y, iy);
-    s.r.lz = __fmul_rd(o4.z, iz);
-    s.r.ux = __fmul_ru(o4.x, ix);
-    s.r.uy = __fmul_ru(o4.y, iy);
-    s.r.uz = __fmul_ru(o4.z, iz);
+    scaled_origin(o4.x, d4.x, ix, s.r.lx, s.r.ux);
+    scaled_origin(o4.y, d4.y, iy, s.r.ly, s.r.uy);
+    scaled_origin(o4.z, d4.z, iz, s.r.lz, s.r.uz);
     s.best_t = s.r.tmax;
     s.best_u = s.best_v = 0.0f;
     s.best_prim = -1;
@@ -362,6 +392,10 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
         float tn0, tf0, tn1, tf1;
         slab(s.r, c.b0, s.tcap, tn0, tf0);
         slab(s.r, c.b1, s.tcap, tn1, tf1);
+        if (flat_ray(s.r)) {
+            slab_flat(s.r, c.b0, s.tcap, tn0, tf0);
+            slab_flat(s.r, c.b1, s.tcap, tn1, tf1);
+        }
         const bool h0 = tn0 <= tf0, h1 = tn1 <= tf1;
         if (h0 && h1) {
             const bool first0 = tn0 <= tn1;

@@ -107,11 +107,8 @@ def test_scene_that_does_not_suit_the_grid(ctx, layout):
     assert (ref["prim"] >= 0).any()
 
 
-@pytest.mark.parametrize("n", [2000, 100_000])
-def test_rays_in_the_planes_of_walls(ctx, n):
-    """Rays that run exactly in the plane of a room's wall, a face of the boxes above it, meet the
-    walls at its ends as the definition says (a slab test that takes 0 times the reciprocal of a
-    zero direction for an exit at t = 0 drops them)."""
+def _rays_in_walls(tmin, tmax):
+    """A room with a few triangles in it, and rays that run exactly in the planes of its walls."""
     box = np.array([[x, y, z] for x in (0, 10) for y in (0, 3) for z in (0, 8)], np.float32)
     quads = [(0, 1, 3, 2), (4, 5, 7, 6), (0, 1, 5, 4), (2, 3, 7, 6), (0, 2, 6, 4), (1, 3, 7, 5)]
     walls = [box[[a, b, c]].reshape(9) for q in quads for a, b, c in (q[:3], (q[0], q[2], q[3]))]
@@ -122,15 +119,42 @@ def test_rays_in_the_planes_of_walls(ctx, n):
     rows = np.arange(2000)
     o[rows, axis] = np.array([10.0, 3.0, 8.0])[axis] * side
     d[rows, axis] = 0.0
-    org = np.concatenate([o, np.full((2000, 1), 1e-4)], 1).astype(np.float32)
-    dir_ = np.concatenate([d, np.full((2000, 1), np.inf)], 1).astype(np.float32)
+    org = np.concatenate([o, np.full((2000, 1), tmin)], 1).astype(np.float32)
+    dir_ = np.concatenate([d, np.full((2000, 1), tmax)], 1).astype(np.float32)
     ref = oracle.trace_brute(tris, org, dir_)
     assert (ref["prim"] >= 0).sum() > 500
+    return tris, org, dir_, ref
+
+
+@pytest.mark.parametrize("n", [2000, 100_000])
+def test_rays_in_the_planes_of_walls(ctx, n):
+    """Rays that run exactly in the plane of a room's wall, a face of the boxes above it, meet the
+    walls at its ends as the definition says (a slab test that takes 0 times the reciprocal of a
+    zero direction for an exit at t = 0 drops them)."""
+    tris, org, dir_, ref = _rays_in_walls(1e-4, np.inf)
     h = hcc.hcc_bvh_upload(ctx, gen.build_bvh(tris), layout="exact")
     try:
         got = _trace(ctx, h, np.tile(org, (n // 2000, 1)), np.tile(dir_, (n // 2000, 1)))
         assert np.array_equal(got.view(np.int32), np.tile(ref, n // 2000).view(np.int32))
     finally:
+        hcc.hcc_bvh_destroy(h)
+
+
+@pytest.mark.parametrize("nodes", ["auto", "layout"])
+@pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
+def test_rays_in_the_planes_of_walls_over_every_node(ctx, nodes, layout):
+    tris, org, dir_, ref = _rays_in_walls(1e-4, np.inf)
+    h = hcc.hcc_bvh_upload(ctx, gen.build_bvh(tris), layout=layout)
+    try:
+        hcc.hcc_set_trace_nodes(ctx, nodes)
+        for schedule in ("auto", "per_ray"):
+            hcc.hcc_set_trace_schedule(ctx, schedule)
+            assert np.array_equal(_trace(ctx, h, org, dir_).view(np.int32), ref.view(np.int32))
+            got = _trace(ctx, h, org, dir_, any_hit=True)
+            assert np.array_equal(got["prim"] >= 0, ref["prim"] >= 0)
+    finally:
+        hcc.hcc_set_trace_nodes(ctx, "auto")
+        hcc.hcc_set_trace_schedule(ctx, "auto")
         hcc.hcc_bvh_destroy(h)
 
 
