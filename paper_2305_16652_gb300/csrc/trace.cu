@@ -32,9 +32,11 @@ namespace {
 
 constexpr int TRACE_BLOCK = 128;
 constexpr int STACK = HCC_TRACE_STACK;
-// 1 + 2 * gamma(3), gamma(n) = n u / (1 - n u), u = 2^-24
-constexpr float ROBUST_FAR = 1.0000003576279f;
-constexpr float PRUNE_SLACK = 1.0f + 1.0f / 65536.0f;
+// What slab distances are widened by, and the best hit before it prunes, as fractions
+// of their magnitudes (distances may be negative): 2 * gamma(3), gamma(n) = n u / (1 - n u),
+// u = 2^-24; and 2^-16.
+constexpr float ROBUST_FAR = 0x3p-23f;
+constexpr float PRUNE_SLACK = 0x1p-16f;
 // idle lanes that make a warp take new rays: in input order, and in sorted
 // order (rays fetched through a permutation), where waiting longer keeps the
 // warp's neighbouring rays together (measured faster for each)
@@ -91,7 +93,7 @@ __device__ __forceinline__ void slab(const Ray &r, const Box2 &b, float tcap, fl
     const float2 z = __fmul2_rn(__fadd2_rn(b.zz, r.nzz), r.izz);
     tn = fmax3(fminf(a.x, c.x), fminf(a.y, c.y), fmaxf(fminf(z.x, z.y), r.tmin));
     const float f = fmin3(fmaxf(a.x, c.x), fmaxf(a.y, c.y), fmaxf(z.x, z.y));
-    tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
+    tf = fminf(__fmaf_rn(fabsf(f), ROBUST_FAR, f), tcap);
 }
 
 // A ray with a zero direction component may lie in the plane of a box's face, where the
@@ -111,7 +113,7 @@ __device__ __forceinline__ void slab_flat(const Ray &r, const Box2 &b, float tca
     const float2 z = __fmul2_rn(__fadd2_rn(b.zz, r.nzz), r.izz);
     tn = fmax3(flat_near(fminf(a.x, c.x)), flat_near(fminf(a.y, c.y)), fmaxf(flat_near(fminf(z.x, z.y)), r.tmin));
     const float f = fmin3(flat_far(fmaxf(a.x, c.x)), flat_far(fmaxf(a.y, c.y)), flat_far(fmaxf(z.x, z.y)));
-    tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
+    tf = fminf(__fmaf_rn(fabsf(f), ROBUST_FAR, f), tcap);
 }
 
 // Moller-Trumbore; returns true with (t, u, v) if the ray's line meets the
@@ -209,7 +211,7 @@ __device__ __forceinline__ float wide_child(const Ray &r, float nx, float ny, fl
     const float ix = r.ixy.x, iy = r.ixy.y, iz = r.izz.x;
     const float tn = fmax3(__fmaf_rd(nx, ix, -r.ux), __fmaf_rd(ny, iy, -r.uy), fmaxf(__fmaf_rd(nz, iz, -r.uz), r.tmin));
     const float f = fmin3(__fmaf_ru(fx, ix, -r.lx), __fmaf_ru(fy, iy, -r.ly), __fmaf_ru(fz, iz, -r.lz));
-    const float tf = fminf(__fmul_rn(f, ROBUST_FAR), tcap);
+    const float tf = fminf(__fmaf_rn(fabsf(f), ROBUST_FAR, f), tcap);
     return (tn <= tf && ref != 0xFFFFFFFFu) ? fminf(tn, 3.40282347e38f) : __int_as_float(0x7F800000);
 }
 
@@ -436,7 +438,7 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
                 s.best_u = u;
                 s.best_v = v;
                 s.best_prim = prim;
-                s.tcap = __fmul_rn(t, PRUNE_SLACK);
+                s.tcap = __fmaf_rn(fabsf(t), PRUNE_SLACK, t);
             }
             hit_any = true;
             if (ANY) break;
@@ -634,7 +636,7 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
 // tau of a hit at t, widened by the prune slack.
 __device__ __forceinline__ float compact_cap(float t, float from, float scale) {
     const float tau = __fsub_ru(t, from);
-    return __fmul_ru(__fmaf_ru(__fadd_ru(fabsf(t), tau), PRUNE_SLACK - 1.0f, tau), scale);
+    return __fmul_ru(__fmaf_ru(__fadd_ru(fabsf(t), tau), PRUNE_SLACK, tau), scale);
 }
 
 // A leaf that is next becomes the lane's parked leaf if it has none (a node of

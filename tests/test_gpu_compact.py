@@ -96,6 +96,21 @@ def test_negative_and_late_intervals(ctx):
 
 
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
+def test_negative_intervals_over_the_layouts_nodes(ctx, layout):
+    """Hits behind the origin, where distances and the best hit are negative."""
+    tris = gen.random_tris(19, 2000, mu=-2.0)
+    org, dir_ = _rays(23, 4000, tris)
+    org[:, 3] = -10.0
+    dir_[::2, 3] = 0.0
+    try:
+        hcc.hcc_set_trace_nodes(ctx, "layout")
+        ref = _check(ctx, tris, org, dir_, layout)
+        assert (ref["t"] < 0).sum() > 200
+    finally:
+        hcc.hcc_set_trace_nodes(ctx, "auto")
+
+
+@pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
 def test_scene_that_does_not_suit_the_grid(ctx, layout):
     """Detail far below the grid's step (a cloud of 1e-6 units in a scene of 1): the layout's nodes are walked."""
     small = (gen.random_tris(29, 300, mu=-1.5) * np.float32(1e-6)).astype(np.float32)
@@ -142,8 +157,9 @@ def test_rays_in_the_planes_of_walls(ctx, n):
 
 @pytest.mark.parametrize("nodes", ["auto", "layout"])
 @pytest.mark.parametrize("layout", ["quantised", "exact", "wide"])
-def test_rays_in_the_planes_of_walls_over_every_node(ctx, nodes, layout):
-    tris, org, dir_, ref = _rays_in_walls(1e-4, np.inf)
+@pytest.mark.parametrize("tmin,tmax", [(1e-4, np.inf), (-50.0, 0.0), (-50.0, np.inf)])
+def test_rays_in_the_planes_of_walls_over_every_node(ctx, nodes, layout, tmin, tmax):
+    tris, org, dir_, ref = _rays_in_walls(tmin, tmax)
     h = hcc.hcc_bvh_upload(ctx, gen.build_bvh(tris), layout=layout)
     try:
         hcc.hcc_set_trace_nodes(ctx, nodes)
