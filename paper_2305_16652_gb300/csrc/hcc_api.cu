@@ -536,7 +536,7 @@ hcc_status hcc_reserve(hcc_ctx *ctx, uint64_t max_n, uint32_t max_key_bits) {
     DeviceGuard g(ctx->device);
     const size_t ksz = max_key_bits > 32 ? 8 : 4;
     hcc_status st;
-    if ((st = ensure(ctx, ctx->sort_scratch, sort_scratch_bytes(max_n, max_key_bits), "sort scratch")) != HCC_OK)
+    if ((st = ensure(ctx, ctx->sort_scratch, sort_scratch_bytes_upto(max_n, max_key_bits), "sort scratch")) != HCC_OK)
         return st;
     if ((st = ensure(ctx, ctx->keys, max_n * ksz, "keys")) != HCC_OK) return st;
     if ((st = ensure(ctx, ctx->perm, max_n * 4, "perm")) != HCC_OK) return st;
@@ -1313,7 +1313,7 @@ hcc_status hcc_sort(hcc_ctx *ctx, const void *keys, uint32_t key_bits, uint64_t 
     const uintptr_t k0 = (uintptr_t)keys, k1 = k0 + n * ksz, p0 = (uintptr_t)perm, p1 = p0 + n * 4;
     if (k0 < p1 && p0 < k1) return fail(ctx, HCC_ERR_INVALID_ARG, "keys and perm overlap");
     DeviceGuard g(ctx->device);
-    hcc_status st = ensure(ctx, ctx->sort_scratch, sort_scratch_bytes(n, key_bits), "sort scratch");
+    hcc_status st = ensure(ctx, ctx->sort_scratch, sort_scratch_bytes_upto(n, key_bits), "sort scratch");
     if (st != HCC_OK) return st;
     cudaError_t e = launch_sort(ctx->stream, keys, key_bits, n, perm, ctx->sort_scratch.p, ctx->d_err, ctx->sort_opt);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "sort launch");

@@ -172,8 +172,10 @@ cudaError_t launch_spawn(cudaStream_t s, const float4 *in_org, const float4 *in_
 cudaError_t launch_key_stats(cudaStream_t s, const void *keys, uint32_t key_bits, const uint32_t *perm, uint64_t n,
                              unsigned long long *cnt);
 
-// Radix sort scratch bytes for n keys of key_bits bits.
+// Radix sort scratch bytes for n keys of key_bits bits, and for any number of
+// keys up to max_n.
 size_t sort_scratch_bytes(uint64_t n, uint32_t key_bits);
+size_t sort_scratch_bytes_upto(uint64_t max_n, uint32_t key_bits);
 
 // Bounded-wait settings of one sort.
 struct SortOptions {

@@ -39,3 +39,30 @@ def test_any_digits_of_64_bit_keys_may_be_equal(ctx, n, bytes_):
         keys &= ~(np.uint64(255) << shift)
         keys |= rng.integers(0, 256, n, dtype=np.uint64) << shift
     assert np.array_equal(gpu_sort(ctx, keys, 64), oracle.stable_sort(keys))
+
+
+@pytest.mark.parametrize("k", [32, 48, 64])
+@pytest.mark.parametrize("reserved,n", [(450_001, 450_000), (460_000, 450_000), (460_000, 420_000), (480_000, 430_000)])
+def test_reserved_scratch_covers_smaller_sorts(k, reserved, n):
+    """The tiles are smaller at 450,000 keys and take more scratch than at somewhat more: a capture, which
+    cannot allocate, of a sort below the reserved size."""
+    rng = np.random.default_rng(n)
+    keys = rng.integers(0, 1 << min(k, 63), n, dtype=np.uint64)
+    dev = torch.from_numpy(keys.astype(np.uint32).view(np.int32) if k <= 32 else keys.view(np.int64)).to("cuda:0")
+    perm = torch.empty(n, dtype=torch.int32, device="cuda:0")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    c = hcc.hcc_create(0, stream)
+    try:
+        hcc.hcc_reserve(c, reserved, k)
+        hcc.hcc_graph_begin(c)
+        try:
+            hcc.hcc_sort(c, dev, k, n, perm)
+        finally:
+            graph = hcc.hcc_graph_end(c)
+        hcc.hcc_graph_launch(c, graph)
+        hcc.hcc_sync(c)
+        assert np.array_equal(perm.cpu().numpy().view(np.uint32), oracle.stable_sort(keys))
+        hcc.hcc_graph_destroy(graph)
+    finally:
+        hcc.hcc_destroy(c)
