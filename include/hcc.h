@@ -129,7 +129,12 @@ hcc_status hcc_create(hcc_ctx **out, int device, void *stream);
 /* Release the context and its scratch after waiting for its stream. */
 hcc_status hcc_destroy(hcc_ctx *ctx);
 
-/* Replace the stream used by later calls. */
+/* Replace the stream used by later calls.  Work queued on the old stream is not
+ * waited for: a call that uses the context's scratch (hcc_sort, hcc_run, hcc_run_host,
+ * hcc_batch_run) must be ordered after such calls on the old one.  Traces
+ * may overlap across a change: each change takes the next of sixteen sets of
+ * trace counters.  A graph keeps those of its capture: its launches must
+ * not overlap one another or traces of the same set. */
 hcc_status hcc_set_stream(hcc_ctx *ctx, void *stream);
 
 /* Pre-allocate sort and pipeline scratch for up to max_n rays and keys of

@@ -42,7 +42,7 @@ struct hcc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     uint32_t *d_err = nullptr;                 // device error word, followed by ...
-    hcc::TraceWork *d_work = nullptr;          // ... the trace's counters
+    uint32_t work_set = 0;                     // ... the traces' counters, of which this set is in use
     hcc_trace_schedule schedule = HCC_TRACE_AUTO;
     hcc_trace_nodes nodes = HCC_TRACE_NODES_AUTO;
     float twopoint_fraction = 0.25f;            // TwoPoint length estimate / largest extent
@@ -354,7 +354,7 @@ void cut_view(const hcc_cut *c, const float4 **boxes, uint32_t *on_device, int *
 // Counters for the persistent trace, or NULL for one thread per ray.
 static TraceWork *trace_work(const hcc_ctx *ctx, int any_hit) {
     const bool refill = ctx->schedule == HCC_TRACE_REFILL || (ctx->schedule == HCC_TRACE_AUTO && !any_hit);
-    return refill ? ctx->d_work : nullptr;
+    return refill ? trace_counters(ctx->d_err, ctx->work_set) : nullptr;
 }
 
 // Stack entries for which a trace may walk compact nodes of depth `stack`: none where the context asks for the layout's.
@@ -424,7 +424,6 @@ hcc_status hcc_create(hcc_ctx **out, int device, void *stream) {
         delete c;
         return HCC_ERR_OOM;
     }
-    c->d_work = trace_counters(c->d_err);
     if (cudaMemset(c->d_err, 0, CTX_WORDS_BYTES) != cudaSuccess) {
         cudaFree(c->d_err);
         delete c;
@@ -525,6 +524,7 @@ hcc_status hcc_destroy(hcc_ctx *ctx) {
 
 hcc_status hcc_set_stream(hcc_ctx *ctx, void *stream) {
     if (!ctx) return HCC_ERR_INVALID_ARG;
+    if (ctx->stream != static_cast<cudaStream_t>(stream)) ctx->work_set = (ctx->work_set + 1) % TRACE_WORKS;
     ctx->stream = static_cast<cudaStream_t>(stream);
     return HCC_OK;
 }

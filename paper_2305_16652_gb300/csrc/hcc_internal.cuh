@@ -200,9 +200,12 @@ struct TraceWork {
     uint32_t done;            // blocks that have finished
     uint32_t pad;
 };
-// A context's device words: the error word, then the trace's counters.
-constexpr size_t CTX_WORDS_BYTES = 16 + sizeof(TraceWork);
-inline TraceWork *trace_counters(uint32_t *err) { return reinterpret_cast<TraceWork *>(err + 4); }
+// A context's device words: the error word, then the traces' counters.  A
+// context takes the next set with every change of its stream, so that traces
+// which overlap there do not share one (a set that two traces share is left non-zero).
+constexpr uint32_t TRACE_WORKS = 16;
+constexpr size_t CTX_WORDS_BYTES = 16 + TRACE_WORKS * sizeof(TraceWork);
+inline TraceWork *trace_counters(uint32_t *err, uint32_t set = 0) { return reinterpret_cast<TraceWork *>(err + 4) + set; }
 
 struct TraceArgs {
     const uint4 *nodes = nullptr;  // 2 (quantised), 4 (exact) or 8 (wide) per node

@@ -325,3 +325,37 @@ def test_small_detail_in_large_scenes_costs_no_more_than_the_layouts_nodes(ctx, 
                 assert t_auto < t_layout
     finally:
         hcc.hcc_bvh_destroy(h)
+
+
+def test_traces_that_overlap_after_a_change_of_stream(ctx):
+    """Each stream's persistent trace hands out every ray, and so do the traces after them."""
+    w = gen.room_workload(1, target_tris=60_000, W=480, H=270, spp=4)
+    n = w.rays.n
+    o, d = torch.from_numpy(w.rays.org).to("cuda:0"), torch.from_numpy(w.rays.dir).to("cuda:0")
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    hits = [torch.empty((n, 4), dtype=torch.int32, device="cuda:0") for _ in range(12)]
+    h = hcc.hcc_bvh_upload(ctx, w.bvh, layout="exact")
+    c = hcc.hcc_create(0, streams[0])
+    try:
+        ref = torch.empty_like(hits[0])
+        hcc.hcc_trace(ctx, h, o, d, ref)
+        hcc.hcc_sync(ctx)
+        for x in hits:
+            x.zero_()
+        torch.cuda.synchronize()
+        for k, x in enumerate(hits):
+            hcc.hcc_set_stream(c, streams[k % 3])
+            hcc.hcc_trace(c, h, o, d, x)
+        torch.cuda.synchronize()
+        hcc.hcc_sync(c)
+        assert all(torch.equal(x, ref) for x in hits)
+        for s in streams:
+            hits[0].zero_()
+            torch.cuda.synchronize()
+            hcc.hcc_set_stream(c, s)
+            hcc.hcc_trace(c, h, o, d, hits[0])
+            hcc.hcc_sync(c)
+            assert torch.equal(hits[0], ref)
+    finally:
+        hcc.hcc_destroy(c)
+        hcc.hcc_bvh_destroy(h)
