@@ -259,7 +259,8 @@ typedef enum hcc_bvh_layout {
  * boxes do not suit them: a scene wider than 1e9 or narrower than 1e-9 units, or
  * detail so small against it that rays about some part of the scene would do a
  * tenth more work plus two node steps (an object of 0.3 units and 130,000
- * triangles: in scenes from 15 units up).
+ * triangles: in scenes from 15 units up).  A BVH that leaves no memory for them
+ * goes without.
  * Traces (single, batches, servers) walk the compact nodes where their deepest
  * stack fits the trace's, unless hcc_set_trace_nodes says otherwise; else they
  * walk the layout's nodes, which are also what hcc_trace_counts counts and what

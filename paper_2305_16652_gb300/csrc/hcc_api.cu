@@ -10,10 +10,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <future>
 #include <new>
 #include <string>
-#include <system_error>
 #include <vector>
 
 #include "hcc_internal.cuh"
@@ -851,7 +851,7 @@ hcc_status hcc_bvh_upload_layout(hcc_ctx *ctx, const hcc_bvh_desc *d, hcc_bvh_la
     std::future<CompactNodes> building;
     try {
         building = std::async(std::launch::async, [&nd, &internal] { return compact_nodes(&nd, (uint32_t)internal.size()); });
-    } catch (const std::system_error &) {  // no thread to be had: built below
+    } catch (const std::exception &) {  // no thread or memory to be had: built below
     }
     std::vector<uint32_t> words;
     uint32_t num_device_nodes = (uint32_t)internal.size();
@@ -920,20 +920,23 @@ hcc_status hcc_bvh_upload_layout(hcc_ctx *ctx, const hcc_bvh_desc *d, hcc_bvh_la
     if (e == cudaSuccess) e = cudaMemcpy(b->d_nodes, words.data(), words.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_tris, tri.data(), tri.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_prim_rec, prim_rec.data(), (size_t)T * 4, cudaMemcpyHostToDevice);
+    // the compact nodes are an addition: a BVH that leaves no memory for them goes without
     CompactNodes compact;
     try {
         compact = building.valid() ? building.get() : compact_nodes(&nd, (uint32_t)internal.size());
     } catch (const std::bad_alloc &) {
-        hcc_bvh_destroy(b);
-        return fail(ctx, HCC_ERR_OOM, "host allocation");
+        compact.usable = false;
     }
-    if (compact.usable) {
-        b->compact_root = compact.root;
-        b->compact_stack = compact.stack;
-        b->grid = compact.grid;
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_compact, compact.words.size() * 4);
-        if (e == cudaSuccess)
+    if (e == cudaSuccess && compact.usable) {
+        if (cudaMalloc(&b->d_compact, compact.words.size() * 4) == cudaSuccess) {
+            b->compact_root = compact.root;
+            b->compact_stack = compact.stack;
+            b->grid = compact.grid;
             e = cudaMemcpy(b->d_compact, compact.words.data(), compact.words.size() * 4, cudaMemcpyHostToDevice);
+        } else {
+            cudaGetLastError();
+            b->d_compact = nullptr;
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
