@@ -678,8 +678,6 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
     const K mask = key_mask<K>(key_bits);
     const uint32_t d = tid & (RADIX - 1), quarter = tid >> 8;
     wait_for_previous();
-    const uint32_t in_key = (uint32_t)__cvta_generic_to_shared(sh.buf[0].key);
-    const uint32_t in_id = (uint32_t)__cvta_generic_to_shared(sh.buf[0].id);
     uint32_t cur = 0;  // the buffer that holds the block's positions; a block alone alternates
     for (uint32_t pass = 0; 8 * pass < key_bits; ++pass) {
         K kreg[SMALL_ITEMS];
@@ -736,40 +734,40 @@ __global__ void __launch_bounds__(SMALL_BLOCK, 1) k_sort_small(const K *__restri
                 if (!PAIRS) sh.buf[cur ^ 1].id[slot] = vreg[i];
             }
         }
-        if (blocks == 1) {  // staged is sorted: no exchange, and the next pass reads it there
+        if (!PAIRS || blocks == 1) {  // staged is sorted: no exchange, and the next pass reads it there
             cur ^= 1;
             __syncthreads();
             continue;
         }
-        cluster_wait();  // every block's counts
-        uint32_t all = 0, before = 0;
-        if (tid < RADIX) {
-            const uint32_t at = (uint32_t)__cvta_generic_to_shared(&sh.count[pass & 1][d]);
-            for (uint32_t r = 0; r < blocks; ++r) {
-                uint32_t v;
-                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_address(at, r)) : "memory");
-                all += v;
-                before += r < rank_in ? v : 0u;
+        if constexpr (PAIRS) {
+            const uint32_t in_key = (uint32_t)__cvta_generic_to_shared(sh.buf[0].key);
+            cluster_wait();  // every block's counts
+            uint32_t all = 0, before = 0;
+            if (tid < RADIX) {
+                const uint32_t at = (uint32_t)__cvta_generic_to_shared(&sh.count[pass & 1][d]);
+                for (uint32_t r = 0; r < blocks; ++r) {
+                    uint32_t v;
+                    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_address(at, r)) : "memory");
+                    all += v;
+                    before += r < rank_in ? v : 0u;
+                }
             }
-        }
-        const uint32_t global = digit_scan(all, sh.wsum[1]);
-        if (tid < RADIX) sh.start[d] = global + before - local;
-        __syncthreads();  // the block's items staged, their global positions ready
+            const uint32_t global = digit_scan(all, sh.wsum[1]);
+            if (tid < RADIX) sh.start[d] = global + before - local;
+            __syncthreads();  // the block's items staged, their global positions ready
 #pragma unroll
-        for (int i = 0; i < SMALL_ITEMS; ++i) {
-            const uint32_t p = tid + (uint32_t)i * SMALL_BLOCK;
-            if (p < tile_n) {
-                const uint64_t e = sh.buf[1].key[p];
-                const uint32_t pos = sh.start[digit_of((K)e, pass)] + p;
-                const uint32_t to = pos / SMALL_CAP, slot = pos % SMALL_CAP;
-                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_address(in_key + slot * 8u, to)), "l"(e) : "memory");
-                if (!PAIRS)
-                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_address(in_id + slot * 4u, to)),
-                                 "r"(sh.buf[1].id[p]) : "memory");
+            for (int i = 0; i < SMALL_ITEMS; ++i) {
+                const uint32_t p = tid + (uint32_t)i * SMALL_BLOCK;
+                if (p < tile_n) {
+                    const uint64_t e = sh.buf[1].key[p];
+                    const uint32_t pos = sh.start[digit_of((K)e, pass)] + p;
+                    const uint32_t to = pos / SMALL_CAP, slot = pos % SMALL_CAP;
+                    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_address(in_key + slot * 8u, to)), "l"(e) : "memory");
+                }
             }
+            cluster_arrive();
+            cluster_wait();  // every item at its place; no block leaves while others may write to it
         }
-        cluster_arrive();
-        cluster_wait();  // every item at its place; no block leaves while others may write to it
     }
     for (uint32_t p = tid; p < tile_n; p += SMALL_BLOCK)
         perm[first + p] = PAIRS ? (uint32_t)(sh.buf[cur].key[p] >> 32) : sh.buf[cur].id[p];
