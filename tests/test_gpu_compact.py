@@ -38,9 +38,10 @@ def _check(ctx, tris, org, dir_, layout="exact"):
         hcc.hcc_bvh_destroy(h)
 
 
-@pytest.mark.parametrize("n", [1, 2, 7, 31, 32, 33, 1000, 38912, 80000, 80001, 155649, 160000])
+@pytest.mark.parametrize("n", [1, 2, 7, 31, 32, 33, 1000, 38912, 50000, 50001, 70000, 70001, 80000, 155649, 160000])
 def test_partial_warps_and_first_refills(ctx, n):
-    """Wavefronts that end inside a warp, and around the first slots taken by refilling."""
+    """Wavefronts that end inside a warp, on both sides of the sizes where four lanes per ray give way
+    to one (50,000 for any hit, 70,000 for closest), and around the first slots taken by refilling."""
     tris = gen.random_tris(3, 60, mu=-1.5)
     org, dir_ = _rays(n, n, tris)
     _check(ctx, tris, org, dir_)

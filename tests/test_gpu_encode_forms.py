@@ -1,6 +1,6 @@
-"""HCC keys where the two-boxes-at-a-time slab test changes form (needs a GB300): odd box
-counts, more than one key word, rays that take the general test beside rays that do not,
-and bounded beside unbounded rays."""
+"""HCC keys where the slab test of the staged boxes changes form (needs a GB300): numbers of boxes
+that the unrolled loop does not divide, both key types, rays that take the general test beside
+rays that do not, and bounded beside unbounded rays."""
 import numpy as np
 import pytest
 

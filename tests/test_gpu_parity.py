@@ -701,12 +701,13 @@ def chunk_room():
     return w
 
 
-# the whole wavefront (chunks of 2^20, 2^21, then 2^22 and the rest), one ray
-# more than a single pass (2^20 + 2^21 + 2^20 + 1), and four chunks with a
-# 5-ray tail
-@pytest.mark.parametrize("n_rays", [None, (1 << 22) + 1, (1 << 20) + (1 << 21) + (1 << 22) + 5])
+# the whole wavefront (a chunk of 2^20, then 2^21 each and the rest); the most rays of
+# a single pass and one more (2^20 + 2^19 + 1); two full chunks, and a third of one
+# ray; and larger counts with tails of 1, 2^20 + 1 and 5 rays
+@pytest.mark.parametrize("n_rays", [None, 3 << 19, (3 << 19) + 1, 3 << 20, (3 << 20) + 1, (5 << 20) + 1, (1 << 22) + 1,
+                                    (7 << 20) + 5])
 def test_run_host_pipeline_over_chunks(ctx, chunk_room, n_rays):
-    """Rays above 2^22 go through the two-stream chunked host pipeline: every
+    """Rays above 1.5 * 2^20 go through the two-stream chunked host pipeline: every
     hit equals the device pipeline's, and a sample equals the oracle's."""
     w = chunk_room
     org_np, dir_np = w.rays.org, w.rays.dir
