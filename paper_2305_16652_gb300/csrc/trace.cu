@@ -497,14 +497,9 @@ struct CompactState {
 
 // Stack slots below the pending subtrees: (tmin, scale) and (from, -), read only when a triangle is met.
 constexpr int COMPACT_SLOTS = 2;
-// relative widening of the exit distance of rays from far outside the scene:
-// the triangle test's own rounding grows with the distance to the origin, as
-// the widening of the other layouts' slab test (ROBUST_FAR) does
-constexpr float FAR_WIDEN = 1.0f / 1048576.0f;
-// ... and its limit, below the gap between the bounds of an unused child: 5.99
-// grid units on the axis that leaves the scene first, whose far side lies at
-// most GRID_REACH + 8 units from the start and at tau 1/4 or more
-constexpr float FAR_WIDEN_MAX = 1.0f / 32.0f;
+// What the triangle test's own rounding may move a ray by, of its distance from its origin
+// (it grows with that distance; the other layouts' slab tests round alike).
+constexpr double FAR_NOISE = 0x1p-20;
 constexpr uint32_t GRID_HI_LO = 0x0220u;  // turns the selector of one bound of a word into the other's
 
 // A 16-bit bound of word w as a grid coordinate in [2, 8): bytes (0, low, high, 0x40).
@@ -512,32 +507,50 @@ __device__ __forceinline__ float grid_bound(uint32_t w, uint32_t sel) {
     return __uint_as_float(__byte_perm(w, 0x40u, sel));
 }
 
-// A ray whose origin is more than GRID_REACH from the grid's zero, or whose
-// interval starts further than that from its origin (tmin far below zero): measures t
-// from the point where it enters the scene's neighbourhood (one unit around the
-// grid's box), computed in double, so that the grid coordinates of the slab test
-// and the distances it takes from them stay small.  Returns false if it never comes near.
-__device__ __noinline__ bool enter_grid(const float4 o4, const float4 d4, const Grid &g, float3 &p, float &from) {
+// A ray as the slab test sees it: point p at t = `from` (to within its rounding), grid-space
+// direction d times 1 / unit, and what its distances may be off by (in t * unit).
+struct GridRay {
+    float3 p, d;
+    float from, unit, noise;
+};
+
+// Sets up, in double, a ray whose origin is more than GRID_REACH from the grid's zero, whose
+// interval starts further than that behind its origin: measures t from the point where it enters the scene's neighbourhood (one
+// unit and the noise around the grid's box), so that the grid coordinates of the slab test
+// and the distances it takes from them stay small, and brings the direction's length near 1.
+// Returns 0 if the ray never comes near, 2 if the noise is larger than the scene on every
+// axis (then no box can be told from any other), else 1.
+__device__ __noinline__ int enter_grid(const float4 o4, const float4 d4, const Grid &g, GridRay &r) {
     const float o[3] = {o4.x, o4.y, o4.z}, d[3] = {d4.x, d4.y, d4.z};
-    double op[3], dp[3], tin = (double)o4.w, tout = (double)d4.w;
+    double op[3], dp[3];
     for (int k = 0; k < 3; ++k) {
         op[k] = ((double)o[k] - (double)g.lo[k]) * (double)g.scale[k] + (double)GRID_ORIGIN;
         dp[k] = (double)d[k] * (double)g.scale[k];
+        if (!isfinite(op[k]) || !isfinite(dp[k])) return 0;  // not a ray
+    }
+    const double longest = fmax(fmax(fabs(dp[0]), fabs(dp[1])), fabs(dp[2]));
+    if (longest == 0.0) return 0;
+    const int e = min(max(ilogb(longest), -120), 120);
+    double tin = (double)o4.w - fabs((double)o4.w) * FAR_NOISE, tout = (double)d4.w + fabs((double)d4.w) * FAR_NOISE;
+    for (int k = 0; k < 3; ++k) {
+        const double lo = 1.0 - fabs(op[k]) * FAR_NOISE, hi = 9.0 + fabs(op[k]) * FAR_NOISE;
         if (dp[k] == 0.0) {
-            if (!(op[k] >= 1.0 && op[k] <= 9.0)) return false;
+            if (!(op[k] >= lo && op[k] <= hi)) return 0;
         } else {
-            const double a = (1.0 - op[k]) / dp[k], b = (9.0 - op[k]) / dp[k];
+            const double a = (lo - op[k]) / dp[k], b = (hi - op[k]) / dp[k];
             tin = fmax(tin, fmin(a, b));
             tout = fmin(tout, fmax(a, b));
         }
     }
-    if (!(tin <= tout)) return false;
-    from = __double2float_rd(tin);
-    p.x = (float)(op[0] + (double)from * dp[0]);
-    p.y = (float)(op[1] + (double)from * dp[1]);
-    p.z = (float)(op[2] + (double)from * dp[2]);
-    // beyond about 10^8 scene sizes `from` no longer resolves the scene
-    return fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)) <= GRID_REACH;
+    if (!(tin <= tout)) return 0;
+    r.from = __double2float_rd(tin);
+    r.unit = (float)scalbn(1.0, e);
+    r.p = make_float3((float)(op[0] + tin * dp[0]), (float)(op[1] + tin * dp[1]), (float)(op[2] + tin * dp[2]));
+    r.d = make_float3((float)scalbn(dp[0], -e), (float)scalbn(dp[1], -e), (float)scalbn(dp[2], -e));
+    r.noise = __double2float_ru(scalbn(fabs(tin) * FAR_NOISE, e));
+    // below the gap between the bounds of an unused child (5.99 units), which must never be met
+    const float slowest = fminf(fminf(fabsf(r.d.x), fabsf(r.d.y)), fabsf(r.d.z));
+    return r.noise * slowest < 5.9f ? 1 : 2;
 }
 
 __device__ __forceinline__ uint32_t local_address(const void *p) {
@@ -583,51 +596,75 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     float3 p = make_float3(__fmaf_rn(__fsub_rn(o4.x, g.lo[0]), g.scale[0], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.y, g.lo[1]), g.scale[1], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.z, g.lo[2]), g.scale[2], GRID_ORIGIN));
-    const float gx = __fmul_rn(d4.x, g.scale[0]), gy = __fmul_rn(d4.y, g.scale[1]), gz = __fmul_rn(d4.z, g.scale[2]);
-    const float ix = grid_inv(gx), iy = grid_inv(gy), iz = grid_inv(gz);
-    float from = o4.w, start = o4.w;  // start: `from` as seen from p
+    float gx = __fmul_rn(d4.x, g.scale[0]), gy = __fmul_rn(d4.y, g.scale[1]), gz = __fmul_rn(d4.z, g.scale[2]);
+    const float longest = fmax3(fabsf(gx), fabsf(gy), fabsf(gz));
+    float from = o4.w, tau_scale;
+    int meets = 1;
+    // the rest for a ray whose tmin is `start` as seen from p and whose distances are off by up to noise
+    auto set_up = [&](float start, float unit, float noise) {
+        const float ix = grid_inv(gx), iy = grid_inv(gy), iz = grid_inv(gz);
+        // the far side of the scene, in t from `from` (times unit)
+        const float cx = __fmaf_rn(-p.x, ix, -start), cy = __fmaf_rn(-p.y, iy, -start), cz = __fmaf_rn(-p.z, iz, -start);
+        const float leave = __fadd_rn(fmin3(__fmaf_rn(ix < 0.0f ? 2.0f : 8.0f, ix, cx), __fmaf_rn(iy < 0.0f ? 2.0f : 8.0f, iy, cy),
+                                            __fmaf_rn(iz < 0.0f ? 2.0f : 8.0f, iz, cz)), noise);
+        const float tmax = __fmaf_ru(__fsub_ru(d4.w, from), unit, noise);
+        // 2^-(e + 2) for a far side in [2^e, 2^(e+1)); a far side at or before the start is a miss
+        const uint32_t e = __float_as_uint(fmaxf(leave, 2e-38f)) >> 23;
+        const float scale = __uint_as_float((252u - (e < 251u ? e : 251u)) << 23);
+        if (!(leave > 0.0f && tmax > 0.0f)) meets = 0;
+        s.ixy = make_float2(__fmul_rn(ix, scale), __fmul_rn(iy, scale));
+        s.iz = __fmul_rn(iz, scale);
+        s.cxy = make_float2(__fmul_rn(cx, scale), __fmul_rn(cy, scale));
+        s.cz = __fmul_rn(cz, scale);
+        // c from the limited reciprocal: the same bits where the limit does not bind, so closest
+        // hits always take it (1080p bounce 3652 us, 3720 behind the branch, by its registers) and
+        // any hit only where it is needed (4.1M shadow rays and their order 556 us, 562 always)
+        if (!ANY || fmax3(fabsf(s.ixy.x), fabsf(s.ixy.y), fabsf(s.iz)) > TAU_INV_MAX) {
+            s.ixy = make_float2(limited_inv(s.ixy.x), limited_inv(s.ixy.y));
+            s.iz = limited_inv(s.iz);
+            const float from_tau = __fmul_rn(-start, scale);
+            s.cxy = make_float2(__fmaf_rn(-p.x, s.ixy.x, from_tau), __fmaf_rn(-p.y, s.ixy.y, from_tau));
+            s.cz = __fmaf_rn(-p.z, s.iz, from_tau);
+        }
+        s.sx = ix < 0.0f ? 0x4325u : 0x4105u;
+        s.sy = iy < 0.0f ? 0x4325u : 0x4105u;
+        s.sz = iz < 0.0f ? 0x4325u : 0x4105u;
+        s.tcap = __fmul_ru(tmax, scale);
+        s.widen = __fmul_rn(noise, scale);
+        tau_scale = __fmul_rn(scale, unit);
+    };
     // (a tmin that far above zero is beyond the scene, and the ray a miss below)
-    const bool far = fmaxf(fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)),
-                           __fmul_rn(-start, fmax3(fabsf(gx), fabsf(gy), fabsf(gz)))) > GRID_REACH;
-    bool meets = true;
-    if (far) {
-        meets = enter_grid(o4, d4, g, p, from);
-        start = 0.0f;
+    if (fmaxf(fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)), __fmul_rn(-from, longest)) > GRID_REACH) {
+        GridRay r = {};
+        meets = enter_grid(o4, d4, g, r);
+        p = r.p;
+        gx = r.d.x;
+        gy = r.d.y;
+        gz = r.d.z;
+        from = r.from;
+        set_up(0.0f, r.unit, r.noise);
+        if (meets == 2) {
+            // every box is met and none is pruned: one axis takes them to entries of at most 3
+            // and exits of at least 2.4 steps, an unused child to 3 and 2.4, the others to 0 and 5.4
+            constexpr float STEP = 1.0f / 16.0f;
+            s.ixy = make_float2(STEP, 0.0f);
+            s.cxy = make_float2(-5.0f * STEP, 0.0f);
+            s.iz = s.cz = 0.0f;
+            s.sx = s.sy = s.sz = 0x4105u;
+            s.widen = 5.4f * STEP;
+            s.tcap = __int_as_float(0x7F800000);
+            from = -__int_as_float(0x7F800000);  // compact_cap: infinite
+            tau_scale = 1.0f;
+        }
+    } else {
+        set_up(from, 1.0f, 0.0f);
     }
-    // the far side of the scene, in t from `from`
-    const float cx = __fmaf_rn(-p.x, ix, -start), cy = __fmaf_rn(-p.y, iy, -start), cz = __fmaf_rn(-p.z, iz, -start);
-    const float leave = fmin3(__fmaf_rn(ix < 0.0f ? 2.0f : 8.0f, ix, cx), __fmaf_rn(iy < 0.0f ? 2.0f : 8.0f, iy, cy),
-                              __fmaf_rn(iz < 0.0f ? 2.0f : 8.0f, iz, cz));
-    const float tmax = __fsub_ru(d4.w, from);
-    // 2^-(e + 2) for a far side in [2^e, 2^(e+1)); a far side at or before the start is a miss
-    const uint32_t e = __float_as_uint(fmaxf(leave, 2e-38f)) >> 23;
-    const float scale = __uint_as_float((252u - (e < 251u ? e : 251u)) << 23);
-    meets = meets && leave > 0.0f && tmax > 0.0f;
-    s.ixy = make_float2(__fmul_rn(ix, scale), __fmul_rn(iy, scale));
-    s.iz = __fmul_rn(iz, scale);
-    s.cxy = make_float2(__fmul_rn(cx, scale), __fmul_rn(cy, scale));
-    s.cz = __fmul_rn(cz, scale);
-    // c from the limited reciprocal: the same bits where the limit does not bind, so closest
-    // hits always take it (1080p bounce 3652 us, 3720 behind the branch, by its registers) and
-    // any hit only where it is needed (4.1M shadow rays and their order 556 us, 562 always)
-    if (!ANY || fmax3(fabsf(s.ixy.x), fabsf(s.ixy.y), fabsf(s.iz)) > TAU_INV_MAX) {
-        s.ixy = make_float2(limited_inv(s.ixy.x), limited_inv(s.ixy.y));
-        s.iz = limited_inv(s.iz);
-        const float from_tau = __fmul_rn(-start, scale);
-        s.cxy = make_float2(__fmaf_rn(-p.x, s.ixy.x, from_tau), __fmaf_rn(-p.y, s.ixy.y, from_tau));
-        s.cz = __fmaf_rn(-p.z, s.iz, from_tau);
-    }
-    s.sx = ix < 0.0f ? 0x4325u : 0x4105u;
-    s.sy = iy < 0.0f ? 0x4325u : 0x4105u;
-    s.sz = iz < 0.0f ? 0x4325u : 0x4105u;
-    s.tcap = __fmul_ru(tmax, scale);
-    s.widen = far ? fminf(__fmul_rn(__fmul_rn(fabsf(from), FAR_WIDEN), scale), FAR_WIDEN_MAX) : 0.0f;
     s.far_cxy = make_float2(__fadd_ru(s.cxy.x, s.widen), __fadd_ru(s.cxy.y, s.widen));
     s.far_cz = __fadd_ru(s.cz, s.widen);
     s.best_t = d4.w;
     s.best_u = s.best_v = 0.0f;
     s.best_prim = -1;
-    stack[0] = make_uint2(__float_as_uint(o4.w), __float_as_uint(scale));
+    stack[0] = make_uint2(__float_as_uint(o4.w), __float_as_uint(tau_scale));
     stack[1] = make_uint2(__float_as_uint(from), 0u);
     s.node = meets ? root : REF_NONE;
     s.leaf = REF_NONE;

@@ -271,6 +271,30 @@ def test_intervals_that_start_far_behind_the_origin(ctx, tmin, size):
     assert (ref["prim"] >= 0).sum() > 300 and (ref["t"] < 0).sum() > 100
 
 
+def _aimed(seed, n, size, distance, length, zeros):
+    """Rays at a scene of `size` units from `distance` scene sizes away, directions of the given length."""
+    rng = np.random.default_rng(seed)
+    o = rng.random((n, 3))
+    d = rng.random((n, 3)) - o
+    axis = rng.integers(0, 3, n)
+    for k in range(zeros):
+        d[np.arange(n), (axis + k) % 3] = 0
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    org = np.concatenate([(o - d * distance) * size, np.zeros((n, 1))], 1).astype(np.float32)
+    return org, np.concatenate([d * length, np.full((n, 1), np.inf)], 1).astype(np.float32)
+
+
+# beyond 10^5 scene sizes the triangle test itself tells apart nothing smaller than the scene's
+# triangles on the axes that a ray moves along, so there only rays along an axis have answers that
+# do not hang on the last bits of every box test; from 10^9 on every triangle is tested
+@pytest.mark.parametrize("distance,zeros", [(1e2, 0), (1e4, 0), (1e9, 0), (1e4, 2), (1e6, 2), (1e7, 2), (1e8, 2), (1e9, 2)])
+def test_rays_from_very_far_away(ctx, distance, zeros):
+    tris = gen.random_tris(73, 600, mu=-1.5)
+    org, dir_ = _aimed(79, 3000, 1.0, distance, 1.0, zeros)
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > (20 if distance == 1e9 and not zeros else 2500)
+
+
 def _trace_us(ctx, h, org, dir_, nodes, any_hit):
     hits = torch.zeros((org.shape[0], 4), dtype=torch.int32, device="cuda:0")
     hcc.hcc_set_trace_nodes(ctx, nodes)
