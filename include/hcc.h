@@ -171,7 +171,8 @@ hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule);
  * fits, else its layout's (see hcc_bvh_layout).  LAYOUT: always its layout's,
  * for programs whose rays are so alike that these stay in L1 (sorted rays off
  * one patch of floor: exact nodes 3 to 14 % faster).  Results do not depend on
- * it, except which hit an any-hit query reports.  Servers use AUTO.
+ * it, except which hit an any-hit query reports and for directions shorter than
+ * 1e-28, which the layout's nodes take for zero.  Servers use AUTO.
  * Errors: INVALID_ARG for another value.
  */
 typedef enum hcc_trace_nodes {

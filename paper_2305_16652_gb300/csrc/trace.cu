@@ -500,6 +500,8 @@ constexpr int COMPACT_SLOTS = 2;
 // What the triangle test's own rounding may move a ray by, of its distance from its origin
 // (it grows with that distance; the other layouts' slab tests round alike).
 constexpr double FAR_NOISE = 0x1p-20;
+// Least component of a direction that counts, of the longest one.
+constexpr float LEAST_COMPONENT = 0x1p-60f;
 constexpr uint32_t GRID_HI_LO = 0x0220u;  // turns the selector of one bound of a word into the other's
 
 // A 16-bit bound of word w as a grid coordinate in [2, 8): bytes (0, low, high, 0x40).
@@ -515,7 +517,8 @@ struct GridRay {
 };
 
 // Sets up, in double, a ray whose origin is more than GRID_REACH from the grid's zero, whose
-// interval starts further than that behind its origin: measures t from the point where it enters the scene's neighbourhood (one
+// interval starts further than that behind its origin, or whose direction is of extreme
+// length: measures t from the point where it enters the scene's neighbourhood (one
 // unit and the noise around the grid's box), so that the grid coordinates of the slab test
 // and the distances it takes from them stay small, and brings the direction's length near 1.
 // Returns 0 if the ray never comes near, 2 if the noise is larger than the scene on every
@@ -549,7 +552,8 @@ __device__ __noinline__ int enter_grid(const float4 o4, const float4 d4, const G
     r.d = make_float3((float)scalbn(dp[0], -e), (float)scalbn(dp[1], -e), (float)scalbn(dp[2], -e));
     r.noise = __double2float_ru(scalbn(fabs(tin) * FAR_NOISE, e));
     // below the gap between the bounds of an unused child (5.99 units), which must never be met
-    const float slowest = fminf(fminf(fabsf(r.d.x), fabsf(r.d.y)), fabsf(r.d.z));
+    const float least = LEAST_COMPONENT * fmax3(fabsf(r.d.x), fabsf(r.d.y), fabsf(r.d.z));
+    const float slowest = fmaxf(fminf(fminf(fabsf(r.d.x), fabsf(r.d.y)), fabsf(r.d.z)), least);
     return r.noise * slowest < 5.9f ? 1 : 2;
 }
 
@@ -560,19 +564,14 @@ __device__ __forceinline__ uint32_t local_address(const void *p) {
 }
 
 // As safe_inv, for a grid-space direction; one ulp of error, which the bounds' margin covers.
-__device__ __forceinline__ float grid_inv(float d) {
+// A component of less than `least` counts as that much: at 2^-60 of the longest one it moves
+// a ray by nothing, and what comes of its reciprocal stays finite at any scale.
+// (A constant least value, of 1e-36, took c to infinity for rays that soon leave the scene.)
+__device__ __forceinline__ float grid_inv(float d, float least) {
     float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) > 1e-36f ? d : copysignf(1e-36f, d)));
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(fabsf(d) > least ? d : copysignf(least, d)));
     return r;
 }
-
-// Reciprocal of a grid-space direction in tau, limited so that its products with
-// grid coordinates (below GRID_REACH) stay finite: for a component that grid_inv replaced, the
-// scale of a ray that leaves the scene soon would take them to infinity, which
-// is neither before nor behind the ray.  At the limit the smallest gap between two bounds
-// is still 1e31 in tau, as wide as an axis that the ray does not move along has to be.
-constexpr float TAU_INV_MAX = 1e36f;
-__device__ __forceinline__ float limited_inv(float inv) { return fminf(fmaxf(inv, -TAU_INV_MAX), TAU_INV_MAX); }
 
 // A lane without a ray.
 __device__ __forceinline__ void ray_none(CompactState &s, uint32_t stack_base) {
@@ -584,7 +583,6 @@ __device__ __forceinline__ bool ray_done(const CompactState &s, uint32_t stack_b
     return s.node == REF_NONE && s.leaf == REF_NONE && s.sp == stack_base;
 }
 
-template <bool ANY>
 __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const float4 o4, const float4 d4,
                                          const Grid &g, uint32_t root) {
     s.ox = o4.x;
@@ -596,13 +594,14 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
     float3 p = make_float3(__fmaf_rn(__fsub_rn(o4.x, g.lo[0]), g.scale[0], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.y, g.lo[1]), g.scale[1], GRID_ORIGIN),
                            __fmaf_rn(__fsub_rn(o4.z, g.lo[2]), g.scale[2], GRID_ORIGIN));
-    float gx = __fmul_rn(d4.x, g.scale[0]), gy = __fmul_rn(d4.y, g.scale[1]), gz = __fmul_rn(d4.z, g.scale[2]);
+    const float gx = __fmul_rn(d4.x, g.scale[0]), gy = __fmul_rn(d4.y, g.scale[1]), gz = __fmul_rn(d4.z, g.scale[2]);
     const float longest = fmax3(fabsf(gx), fabsf(gy), fabsf(gz));
     float from = o4.w, tau_scale;
     int meets = 1;
     // the rest for a ray whose tmin is `start` as seen from p and whose distances are off by up to noise
-    auto set_up = [&](float start, float unit, float noise) {
-        const float ix = grid_inv(gx), iy = grid_inv(gy), iz = grid_inv(gz);
+    auto set_up = [&](float3 dir, float length, float start, float unit, float noise) {
+        const float least = __fmul_rn(length, LEAST_COMPONENT);
+        const float ix = grid_inv(dir.x, least), iy = grid_inv(dir.y, least), iz = grid_inv(dir.z, least);
         // the far side of the scene, in t from `from` (times unit)
         const float cx = __fmaf_rn(-p.x, ix, -start), cy = __fmaf_rn(-p.y, iy, -start), cz = __fmaf_rn(-p.z, iz, -start);
         const float leave = __fadd_rn(fmin3(__fmaf_rn(ix < 0.0f ? 2.0f : 8.0f, ix, cx), __fmaf_rn(iy < 0.0f ? 2.0f : 8.0f, iy, cy),
@@ -616,16 +615,6 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
         s.iz = __fmul_rn(iz, scale);
         s.cxy = make_float2(__fmul_rn(cx, scale), __fmul_rn(cy, scale));
         s.cz = __fmul_rn(cz, scale);
-        // c from the limited reciprocal: the same bits where the limit does not bind, so closest
-        // hits always take it (1080p bounce 3652 us, 3720 behind the branch, by its registers) and
-        // any hit only where it is needed (4.1M shadow rays and their order 556 us, 562 always)
-        if (!ANY || fmax3(fabsf(s.ixy.x), fabsf(s.ixy.y), fabsf(s.iz)) > TAU_INV_MAX) {
-            s.ixy = make_float2(limited_inv(s.ixy.x), limited_inv(s.ixy.y));
-            s.iz = limited_inv(s.iz);
-            const float from_tau = __fmul_rn(-start, scale);
-            s.cxy = make_float2(__fmaf_rn(-p.x, s.ixy.x, from_tau), __fmaf_rn(-p.y, s.ixy.y, from_tau));
-            s.cz = __fmaf_rn(-p.z, s.iz, from_tau);
-        }
         s.sx = ix < 0.0f ? 0x4325u : 0x4105u;
         s.sy = iy < 0.0f ? 0x4325u : 0x4105u;
         s.sz = iz < 0.0f ? 0x4325u : 0x4105u;
@@ -633,16 +622,15 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
         s.widen = __fmul_rn(noise, scale);
         tau_scale = __fmul_rn(scale, unit);
     };
-    // (a tmin that far above zero is beyond the scene, and the ray a miss below)
-    if (fmaxf(fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z)), __fmul_rn(-from, longest)) > GRID_REACH) {
+    // a far origin or a direction longer than 2^120, a far tmin behind the origin (one that far
+    // ahead is beyond the scene, and the ray a miss above), or a direction shorter than 2^-60
+    if (fmax3(__fmaf_rn(longest, 0x1p-115f, fmax3(fabsf(p.x), fabsf(p.y), fabsf(p.z))), __fmul_rn(-from, longest),
+              __fmaf_rn(longest, -0x1p70f, 0x1p10f)) > GRID_REACH) {
         GridRay r = {};
         meets = enter_grid(o4, d4, g, r);
         p = r.p;
-        gx = r.d.x;
-        gy = r.d.y;
-        gz = r.d.z;
         from = r.from;
-        set_up(0.0f, r.unit, r.noise);
+        set_up(r.d, fmax3(fabsf(r.d.x), fabsf(r.d.y), fabsf(r.d.z)), 0.0f, r.unit, r.noise);
         if (meets == 2) {
             // every box is met and none is pruned: one axis takes them to entries of at most 3
             // and exits of at least 2.4 steps, an unused child to 3 and 2.4, the others to 0 and 5.4
@@ -657,7 +645,7 @@ __device__ __forceinline__ void ray_init(CompactState &s, uint2 *stack, const fl
             tau_scale = 1.0f;
         }
     } else {
-        set_up(from, 1.0f, 0.0f);
+        set_up(make_float3(gx, gy, gz), longest, from, 1.0f, 0.0f);
     }
     s.far_cxy = make_float2(__fadd_ru(s.cxy.x, s.widen), __fadd_ru(s.cxy.y, s.widen));
     s.far_cz = __fadd_ru(s.cz, s.widen);
@@ -922,7 +910,7 @@ __device__ __forceinline__ bool start_ray(const TraceArgs &a, uint64_t i, State 
         nodes = LAYOUT == COMPACT ? sc->cnodes : sc->nodes;
     }
     if constexpr (LAYOUT == COMPACT) {
-        ray_init<ANY>(s, stack, o4, d4, MULTI ? sc->grid : a.grid, MULTI ? sc->croot : a.croot);
+        ray_init(s, stack, o4, d4, MULTI ? sc->grid : a.grid, MULTI ? sc->croot : a.croot);
         if (!ANY) s.tcap = fminf(s.tcap, CAP_MAX);
     } else {
         ray_init(s, o4, d4, MULTI ? sc->root_ref : a.root_ref);

@@ -295,6 +295,16 @@ def test_rays_from_very_far_away(ctx, distance, zeros):
     assert (ref["prim"] >= 0).sum() > (20 if distance == 1e9 and not zeros else 2500)
 
 
+@pytest.mark.parametrize("size,length", [(1.0, 1e-36), (1.0, 1e-34), (1.0, 1e-19), (1.0, 1e-17), (1.0, 1e30), (1.0, 1e38),
+                                         (1e8, 1e-28), (1e8, 1e-20), (1e-8, 1e20), (1e-3, 1e28), (1e-3, 1e37)])
+@pytest.mark.parametrize("zeros", [0, 1])
+def test_direction_lengths_at_the_ends_of_the_range(ctx, size, length, zeros):
+    tris = (gen.random_tris(83, 600, mu=-1.5) * np.float32(size)).astype(np.float32)
+    org, dir_ = _aimed(89, 3000, size, 0.5, length, zeros)
+    ref = _check(ctx, tris, org, dir_)
+    assert (ref["prim"] >= 0).sum() > 2500
+
+
 def _trace_us(ctx, h, org, dir_, nodes, any_hit):
     hits = torch.zeros((org.shape[0], 4), dtype=torch.int32, device="cuda:0")
     hcc.hcc_set_trace_nodes(ctx, nodes)
