@@ -169,8 +169,8 @@ hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule);
  * Nodes that the context's traces walk, single wavefronts and batches.  AUTO
  * (the default): the compact nodes where the BVH has them and its deepest stack
  * fits, else its layout's (see hcc_bvh_layout).  LAYOUT: always its layout's,
- * for programs whose rays are so alike that these stay in L1 (sorted rays off
- * one patch of floor: exact nodes 3 to 14 % faster).  Results do not depend on
+ * for programs whose rays are so alike that these stay in L1 (rays off one
+ * patch of floor sorted by origin and direction: exact nodes 10 % faster).  Results do not depend on
  * it, except which hit an any-hit query reports and for directions shorter than
  * 1e-28, which the layout's nodes take for zero.  Servers use AUTO.
  * Errors: INVALID_ARG for another value.
@@ -269,7 +269,8 @@ typedef enum hcc_bvh_layout {
 
 /* hcc_bvh_upload with a choice of node layout.  Every layout gives the same
  * hits (boxes only decide which triangles are tested, and every box holds
- * the exact box of its BVH2 node); the quantised one halves node memory, the
+ * the exact box of its BVH2 node); the quantised one's nodes take half the
+ * memory of the exact one's (the compact nodes come on top of either), the
  * exact one avoids decoding work per node visit, and the wide one visits
  * about half as many nodes per ray.  Cuts are always chosen on the BVH2.
  * Errors: as hcc_bvh_upload, plus INVALID_ARG for an unknown layout. */

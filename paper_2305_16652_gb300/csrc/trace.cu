@@ -14,7 +14,9 @@
 // nodes' directed-rounding distances leave only the reciprocal's rounding
 // to cover, the compact nodes' bounds hold a margin for it), and a subtree is dropped only when its entry
 // distance exceeds the best hit by more than 2^-16 relative, so traversal
-// never loses a triangle that the closest-hit definition would pick.
+// reaches every triangle that a ray meets.  (One that only the rounding of the
+// triangle test lets it meet, past an edge or from 10^5 scene sizes away, may
+// lie outside the boxes on the way to it.)
 // Triangle arithmetic is the canonical Moller-Trumbore sequence with explicit
 // round-to-nearest intrinsics (built with --fmad=false), so the (t, u, v) of
 // a triangle are the same bit patterns on every run and in every ray order.
@@ -1276,8 +1278,9 @@ cudaError_t launch_layout(cudaStream_t s, const TraceArgs &a, bool pool) {
     // against compact: the room's 16.6M rays unsorted 4.79 -> 3.00 ms, in HCC order
     // 3.97 -> 2.92, 33.2M shadow rays 3.82 -> 3.18 and 2.90 -> 2.49).  Rays so alike
     // that the binary nodes stay in L1 gain least, as a step over four children is
-    // bound by its arithmetic: 16.6M rays off one patch of floor 3.76 -> 3.25 ms
-    // unsorted, but 3.01 -> 3.11 in HCC order and 2.63 -> 3.00 by origin and direction.
+    // bound by its arithmetic: 16.6M rays off one patch of floor 3.75 -> 3.20 ms
+    // unsorted, but 3.04 -> 3.06 in HCC order and 2.67 -> 2.95 by origin and direction
+    // (a context may ask for its layout's nodes: a.cstack is then beyond any stack).
     if constexpr (!CNT) {
         const int depth = pool && !ANY ? a.stack : STACK;
         if (a.cstack <= (uint32_t)depth) {
