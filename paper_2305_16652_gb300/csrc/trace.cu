@@ -468,8 +468,8 @@ __device__ __forceinline__ void ray_round(RayState &s, uint2 *stack, const uint4
 // instruction.  A compact node is read with two 32-byte loads for four children, so a
 // ray needs 16 visits and 33 loads where the binary nodes take 36 and 72, and the room's
 // nodes shrink from 32 to 13 MB.  What bounds the walk now (ncu, 1.0M rays in
-// HCC order): the ALU pipe 63 %, issue 62 %, L1 data pipe 61 % busy at 21 lanes an
-// instruction, waits for loads 4.4 of 12.3 cycles per instruction; for 16.6M rays
+// HCC order): the ALU pipe 64 %, issue 62 %, L1 data pipe 60 % busy at 21 lanes an
+// instruction, waits for loads 4.3 of 12.2 cycles per instruction; for 16.6M rays
 // 2.45 billion warp instructions against 3.41.
 
 // Traversal state over compact 4-ary nodes.  The slab test works in the
