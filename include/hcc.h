@@ -170,9 +170,11 @@ hcc_status hcc_set_trace_schedule(hcc_ctx *ctx, hcc_trace_schedule schedule);
  * (the default): the compact nodes where the BVH has them and its deepest stack
  * fits, else its layout's (see hcc_bvh_layout).  LAYOUT: always its layout's,
  * for programs whose rays are so alike that these stay in L1 (rays off one
- * patch of floor sorted by origin and direction: exact nodes 10 % faster).  Results do not depend on
- * it, except which hit an any-hit query reports and for directions shorter than
- * 1e-28, which the layout's nodes take for zero.  Servers use AUTO.
+ * patch of floor sorted by origin and direction: exact nodes 10 % faster).
+ * Results do not depend on it, except which hit an any-hit query reports, hits
+ * within rounding of a triangle's edge (where the edge is also one of its box),
+ * and directions shorter than 1e-28, which the layout's nodes take for zero.
+ * Servers use AUTO.
  * Errors: INVALID_ARG for another value.
  */
 typedef enum hcc_trace_nodes {
